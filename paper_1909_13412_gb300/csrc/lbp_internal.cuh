@@ -226,6 +226,17 @@ __device__ __forceinline__ float fix_to_float(long long a) {
     return a < 0 ? -f : f;
 }
 
+// The exact FP64 value of a float, formed from its bits: the conversion
+// instruction occupies the FP64 pipe.  A normal number's exponent is rebiased
+// and its mantissa split over the two words; denormals, infinities and NaNs
+// take the instruction.
+__device__ __forceinline__ double widen_f32(float v) {
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    return m == 0u ? __hiloint2double((int)b, 0) : (double)v;
+}
+
 // Reaction forces are summed per node in 64-bit fixed point so that the sum
 // is exact and independent of the order in which particles add to it.
 constexpr double FIX_SCALE = 72057594037927936.0;  // 2^56
@@ -329,7 +340,7 @@ struct RepTable {
     Rep rep[MAXR];
 };
 
-// replica of a block / of a global node: last r with off[r] <= v (uniform per block)
+// replica of a block: last r with item_off[r] <= b (uniform per block)
 template <int MAXR>
 __device__ __forceinline__ int find_block_rep(const RepTable<MAXR> &t, unsigned b) {
     if (MAXR == 1) return 0;
@@ -337,17 +348,6 @@ __device__ __forceinline__ int find_block_rep(const RepTable<MAXR> &t, unsigned 
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (t.item_off[mid] <= b) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-template <int MAXR>
-__device__ __forceinline__ int find_node_rep(const RepTable<MAXR> &t, long long node) {
-    if (MAXR == 1) return 0;
-    int lo = 0, hi = t.nrep - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (t.rep[mid].node_off <= node) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
