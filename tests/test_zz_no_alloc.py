@@ -106,3 +106,25 @@ def test_noalloc_vacf_rejects_sizes_beyond_its_scratch():
                                                ctypes.c_void_p(cnt.data_ptr()), ctypes.c_void_p(0))
     assert st == lbp.LBP_EINVAL
     assert "scratch" in lbp.lbp_last_error()
+
+
+@pytest.mark.parametrize("T,ncomp,K,offset", [
+    (1, 1, 0, 0), (63, 3, 200, 0), (64, 65, 127, 0), (65, 64, 128, 0), (129, 132, 130, 1), (300, 7, 129, 0),
+    (1000, 1030, 260, 0), (70, 12, 524287, 0), (4000, 2, 255, 0)])
+def test_noalloc_vacf_at_the_edges_of_its_tiles(T, ncomp, K, offset):
+    """Sizes around 64 samples, 64 components and 128 lags; lags past the
+    trajectory; rows that are not 16-byte aligned; the whole scratch in one run.
+    Against the FP64 sums: a block's products of one component are a chain of at
+    most 64 FP32 FMAs, so |error| <= 64 2^-24 sum |x(t) x(t + k)|."""
+    g = np.random.default_rng([T, ncomp, K])
+    x = (g.standard_normal((T, ncomp)) * 0.01).astype(np.float32)
+    flat = torch.zeros(T * ncomp + offset, dtype=torch.float32, device="cuda")
+    flat[offset:] = torch.from_numpy(x.reshape(-1)).cuda()
+    got, cnt = _noalloc(flat[offset:], T, ncomp, K, 5)
+    y = x.astype(np.float64)
+    for k in list(range(0, min(K, T - 1) + 1, max(1, K // 300))) + [min(K, T - 1)]:
+        terms = y[:T - k] * y[k:]
+        assert abs(got[k] - terms.sum()) <= 64 * 2.0 ** -24 * np.abs(terms).sum(), k
+    k = np.arange(K + 1)
+    assert np.array_equal(cnt, np.where(k < T, 5 * (T - k), 0))
+    assert not got[T:].any()
