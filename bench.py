@@ -450,7 +450,7 @@ def run_gpu(args, w):
 
     def timed(h, wk, steps, warmup, clocks=None):
         """K steps between CUDA events on the caller's stream, on the path users
-        run (CUDA-graph replay, no per-launch events), with the VACF blocks of the
+        run (chained launches, no per-launch events), with the VACF blocks of the
         timed samples -- including the last, partial one, flushed before the end
         event -- inside the region.  Then the same K steps once more with the
         library's events around every stream-collide launch, for that kernel's
@@ -615,7 +615,7 @@ def run_gpu(args, w):
         # block at the end of the region
         "gpu_launches": LAUNCHES_PER_STEP * args.steps
                         + (1 if isinstance(w, wl.Ensemble) else VACF_LAUNCHES) * (args.steps // 64 + 1),
-        "timing": "headline on the graph-replay path without per-launch events; the lattice "
+        "timing": "headline on the chained-launch path without per-launch events; the lattice "
                   "kernel's average from a second, instrumented pass of the same steps",
         "clocks": clk.summary(),
     }

@@ -203,12 +203,11 @@ lbp_status lbp_step(lbp_sim *sim, int64_t nsteps);
  * and velocities after it (as lbp_particles_read).  The call returns when the
  * host outputs are written (on_device = 0) or, for device pointers, with the
  * work queued on the handle's stream.
- * With graphs on and 8-byte aligned buffers that the device can address --
+ * With 8-byte aligned buffers that the device can address --
  * memory of the current device (on_device = 1), or page-locked host memory
  * mapped into the device's address space (cudaHostAlloc / cudaHostRegister
  * with unified addressing) -- the step's particle kernel itself reads f_ext
- * and writes r and v, and the step replays as one CUDA graph per buffer
- * parity, cached on the three buffer addresses.  For host buffers, positions
+ * and writes r and v.  For host buffers, positions
  * and velocities are final after the particle kernel (Eqs. 1-2), whose last
  * block then sets a completion flag in page-locked memory, so the call
  * returns (after a bounded poll of that flag: LBP_ECUDA or LBP_ETIMEOUT if
@@ -382,7 +381,10 @@ lbp_status lbp_autotune(lbp_sim *sim, int launches, int *rows, int *variant, dou
 lbp_status lbp_set_block_shape(lbp_sim *sim, int rows, int variant);
 lbp_status lbp_set_block_rows(lbp_sim *sim, int rows);
 
-/* Use CUDA graphs for lbp_step (default 1).                                  */
+/* How the kernels of one call's steps are launched; results do not depend on
+ * it.  1 (default): as a chain, each kernel the programmatic dependent of the
+ * one before, so that launches overlap; 0: only a step's lattice pass on its
+ * particle kernel.  (The name is from when the chain was a CUDA graph per step.)  */
 lbp_status lbp_set_use_graphs(lbp_sim *sim, int enable);
 
 /* Kernel timing: while enabled, lbp_step records CUDA events around every

@@ -8,8 +8,10 @@
 //      s1:  after every 64th step the VACF block, which overlaps the next
 //           steps; s0 waits for it only before the following block is forked.
 //
-// A step is captured into a CUDA graph per buffer parity and replayed; the
-// VACF fork stays outside the graph.
+// The kernels of the steps of one call are launched as a chain of programmatic
+// dependents (grid_dependency_wait in lbp_internal.cuh), not as replayed CUDA
+// graphs: a graph of one step measured the same per step as its two launches
+// (14.35 us at 32^3 both), and between graphs the chain is cut.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -89,19 +91,6 @@ lbp_status leave(lbp_sim *s) {
     return LBP_OK;
 }
 
-void drop_graphs(lbp_sim *s) {
-    for (int i = 0; i < 2; ++i) {
-        if (s->graph[i]) {
-            cudaGraphExecDestroy(s->graph[i]);
-            s->graph[i] = nullptr;
-        }
-        if (s->xgraph[i]) {
-            cudaGraphExecDestroy(s->xgraph[i]);
-            s->xgraph[i] = nullptr;
-        }
-    }
-}
-
 lbp_status stage(lbp_sim *s, size_t bytes) {
     if (s->stage_bytes >= bytes) return LBP_OK;
     if (s->stage) {
@@ -140,13 +129,15 @@ double nu_of(double tau) { return (tau - 0.5) / 3.0; }
 // buffers of lbp_step_exchange: device buffers, or the device views of
 // page-locked host buffers) the particle kernel reads the external forces and
 // writes the positions and velocities itself, and for host buffers raises the
-// step's completion flag.
-lbp_status enqueue_step(lbp_sim *s, bool timed, const ParticleIO *io = nullptr) {
+// step's completion flag.  `chained`: the previous launch on s0 was the lattice
+// pass of the step before, of which the particle kernel becomes the
+// programmatic dependent.
+lbp_status enqueue_step(lbp_sim *s, bool timed, bool chained, const ParticleIO *io) {
     Range range("lbp step: particles + lattice pass");
     const void *src = s->f[s->cur];
     void *dst = s->f[s->cur ^ 1];
     const int parity = s->cur;
-    if (s->np > 0) CK(launch_particles(*s, src, parity, s->s0, io));
+    if (s->np > 0) CK(launch_particles(*s, src, parity, s->s0, io, chained));
     if (timed) CK(cudaEventRecord(s->tev[2 * s->ntimed], s->s0));
     // the lattice pass as the programmatic dependent of the particle kernel
     // (its population loads overlap the particle kernel's tail); not when
@@ -198,29 +189,10 @@ lbp_status fold_timing(lbp_sim *s) {
     return LBP_OK;
 }
 
-lbp_status capture(lbp_sim *s, int parity) {
-    cudaGraph_t g = nullptr;
-    const int saved = s->cur;
-    s->cur = parity;
-    CK(cudaStreamBeginCapture(s->s0, cudaStreamCaptureModeThreadLocal));
-    lbp_status st = enqueue_step(s, false);
-    cudaError_t e = cudaStreamEndCapture(s->s0, &g);
-    s->cur = saved;
-    if (st != LBP_OK) {
-        if (g) cudaGraphDestroy(g);
-        return st;
-    }
-    CK(e);
-    e = cudaGraphInstantiate(&s->graph[parity], g, 0);
-    cudaGraphDestroy(g);
-    CK(e);
-    return LBP_OK;
-}
-
-// one time step on s0 (graph replay, timed or plain launches); `whole`, when
-// given, is a graph that holds this step with its host exchange and replaces
-// the step graph of this parity
-lbp_status step_once(lbp_sim *s, cudaGraphExec_t whole = nullptr) {
+// one time step on s0.  `follows`: the last thing queued on s0 is the lattice
+// pass of the step before (within one call), so the two can be chained; on
+// return it says the same for the next step.
+lbp_status step_once(lbp_sim *s, bool &follows, const ParticleIO *io = nullptr) {
     // the VACF correlator runs when the step completes a block of B samples
     const int B = vacf_block_samples();
     bool due = false;
@@ -231,17 +203,10 @@ lbp_status step_once(lbp_sim *s, cudaGraphExec_t whole = nullptr) {
             s->vacf_done_host += B;
         }
     }
-    if (whole) {
-        CK(cudaGraphLaunch(whole, s->s0));
-    } else if (s->timing) {
-        if (s->ntimed == lbp::Sim::MAX_TIMED) TRY(fold_timing(s));
-        TRY(enqueue_step(s, true));
-    } else if (s->use_graphs) {
-        if (!s->graph[s->cur]) TRY(capture(s, s->cur));
-        CK(cudaGraphLaunch(s->graph[s->cur], s->s0));
-    } else {
-        TRY(enqueue_step(s, false));
-    }
+    const bool timed = s->timing != 0;
+    if (timed && s->ntimed == lbp::Sim::MAX_TIMED) TRY(fold_timing(s));
+    TRY(enqueue_step(s, timed, follows && !timed && s->chain && lattice_chains(*s), io));
+    follows = !due;
     if (due) TRY(fork_vacf(s));
     s->cur ^= 1;
     s->step += 1;
@@ -250,7 +215,7 @@ lbp_status step_once(lbp_sim *s, cudaGraphExec_t whole = nullptr) {
 
 // the exchange's copies and conversions before and after one step, on s0, for
 // buffers the particle kernel cannot address directly (pageable, another
-// device's, not 8-byte aligned); the others take exchange_graph
+// device's, not 8-byte aligned); the particle kernel does the others' itself
 lbp_status exchange_in(lbp_sim *s, const double *f_ext, cudaMemcpyKind kind) {
     const int n = s->np;
     if (n > 0 && f_ext) {
@@ -282,53 +247,29 @@ lbp_status device_view(double *&p) {
     return LBP_OK;
 }
 
-// [forces in, step, positions and velocities out] from and to page-locked host
-// buffers or device buffers as one graph for the current buffer parity, kept
-// while the same buffers come back: the particle kernel reads and writes the
-// buffers directly, so the graph holds the step's two kernels only
-lbp_status exchange_graph(lbp_sim *s, const double *f_ext, double *r, double *v, int on_device,
-                          cudaGraphExec_t *out) {
-    const int par = s->cur;
-    const void *key[3] = {f_ext, r, v};
-    bool same = s->xgraph[par] && s->xkey_np[par] == s->np && s->xkey_dev[par] == on_device;
-    for (int k = 0; k < 3 && same; ++k) same = s->xkey[par][k] == key[k];
-    if (!same) {
-        if (s->xgraph[par]) {
-            cudaGraphExecDestroy(s->xgraph[par]);
-            s->xgraph[par] = nullptr;
-        }
-        if (!on_device && !s->d_xticket) {
+// one step whose particle kernel reads the forces from, and writes positions and
+// velocities to, page-locked host buffers or device buffers
+lbp_status exchange_step(lbp_sim *s, const double *f_ext, double *r, double *v, int on_device) {
+    double *f_dev = const_cast<double *>(f_ext), *r_dev = r, *v_dev = v;
+    if (!on_device) {
+        if (!s->d_xticket) {
             TRY(dalloc(&s->d_xticket, 1));
-            CK(cudaMemset(s->d_xticket, 0, sizeof(unsigned)));
+            CK(cudaMemsetAsync(s->d_xticket, 0, sizeof(unsigned), s->s0));
+        }
+        if (!s->h_xflag) {
             CK(cudaHostAlloc((void **)&s->h_xflag, sizeof(long long), cudaHostAllocMapped));
-            *s->h_xflag = -1;
             CK(cudaHostGetDevicePointer((void **)&s->h_xflag_dev, s->h_xflag, 0));
         }
-        double *f_dev = const_cast<double *>(f_ext), *r_dev = r, *v_dev = v;
-        if (!on_device) {
-            TRY(device_view(f_dev));
-            TRY(device_view(r_dev));
-            TRY(device_view(v_dev));
-        }
-        cudaGraph_t g = nullptr;
-        CK(cudaStreamBeginCapture(s->s0, cudaStreamCaptureModeThreadLocal));
-        const ParticleIO io{f_dev, r_dev, v_dev, !on_device};
-        lbp_status st = enqueue_step(s, false, &io);
-        cudaError_t e = cudaStreamEndCapture(s->s0, &g);
-        if (st != LBP_OK) {
-            if (g) cudaGraphDestroy(g);
-            return st;
-        }
-        CK(e);
-        e = cudaGraphInstantiate(&s->xgraph[par], g, 0);
-        cudaGraphDestroy(g);
-        CK(e);
-        for (int k = 0; k < 3; ++k) s->xkey[par][k] = key[k];
-        s->xkey_np[par] = s->np;
-        s->xkey_dev[par] = on_device;
+        TRY(device_view(f_dev));
+        TRY(device_view(r_dev));
+        TRY(device_view(v_dev));
+        // the flag may hold this step index from before a lbp_set_step_index or a
+        // checkpoint load; the previous call's kernel has finished writing it
+        __atomic_store_n(s->h_xflag, -1ll, __ATOMIC_RELEASE);
     }
-    *out = s->xgraph[par];
-    return LBP_OK;
+    const ParticleIO io{f_dev, r_dev, v_dev, !on_device};
+    bool follows = false;
+    return step_once(s, follows, &io);
 }
 
 // Wait until the particle kernel of step `step` has written the positions and
@@ -535,7 +476,6 @@ lbp_status lbp_destroy(lbp_sim *s) {
     if (!s) return LBP_OK;
     if (s->s0) cudaStreamSynchronize(s->s0);
     if (s->s1) cudaStreamSynchronize(s->s1);
-    drop_graphs(s);
     free_tape(s);
     void *bufs[] = {s->f[0], s->f[1], s->d_step, s->d_err, s->r, s->v, s->fh, s->fr, s->fext, s->xbuf,
                     s->mass, s->inv_mass, s->gamma, s->radius, s->sig, s->pinned, s->prep, s->fq, s->rec[0],
@@ -782,7 +722,6 @@ lbp_status lbp_particles_add_to(lbp_sim *s, int replica, int n, const double *r,
     s->np = np_new;
     // the VACF ring is laid out per particle count: adding particles turns it off
     s->vacf_lag = -1;
-    drop_graphs(s);
     return leave(s);
 }
 
@@ -861,7 +800,6 @@ lbp_status lbp_particles_set_params(lbp_sim *s, const lbp_particle_params *prm) 
         CK(cudaMemcpyAsync(s->sig, sg.data(), sizeof(double) * s->np, cudaMemcpyHostToDevice, s->s0));
         CK(cudaStreamSynchronize(s->s0));
     }
-    drop_graphs(s);
     return leave(s);
 }
 
@@ -973,7 +911,8 @@ lbp_status lbp_step(lbp_sim *s, int64_t nsteps) {
     if (nsteps < 0) return fail(LBP_EINVAL, "lbp_step: nsteps < 0");
     if (nsteps == 0) return LBP_OK;
     TRY(enter(s));
-    for (int64_t n = 0; n < nsteps; ++n) TRY(step_once(s));
+    bool follows = false;
+    for (int64_t n = 0; n < nsteps; ++n) TRY(step_once(s, follows));
     return leave(s);
 }
 
@@ -989,40 +928,28 @@ lbp_status lbp_step_exchange(lbp_sim *s, const double *f_ext, double *r, double 
             if (s->xbuf) cudaFree(s->xbuf);
             s->xbuf = nullptr;
             s->xbuf_cap = 0;
-            drop_graphs(s);  // the particle capacity grew: captured anew
             TRY(dalloc(&s->xbuf, (size_t)9 * s->cap));
             s->xbuf_cap = s->cap;
         }
     }
     if (n > 0 && f_ext) s->edits += 1;  // as lbp_particles_set_external_force
-    const bool as_graph = n > 0 && s->use_graphs && !s->timing &&
-                          (on_device ? device_memory(f_ext) && device_memory(r) && device_memory(v)
-                                     : host_pinned(f_ext) && host_pinned(r) && host_pinned(v));
-    if (as_graph && on_device) {
-        // the particle kernel reads f_ext and writes r, v in device memory;
-        // stream-ordered like any other step
-        cudaGraphExec_t whole = nullptr;
-        TRY(exchange_graph(s, f_ext, r, v, 1, &whole));
-        TRY(step_once(s, whole));
-        return leave(s);
-    }
-    if (as_graph) {
-        // returns once f_ext has been consumed and r, v are on the host; the
-        // step's lattice pass may still run, and later work on s0 follows it
-        cudaGraphExec_t whole = nullptr;
-        TRY(exchange_graph(s, f_ext, r, v, 0, &whole));
+    const bool direct = n > 0 && !s->timing &&
+                        (on_device ? device_memory(f_ext) && device_memory(r) && device_memory(v)
+                                   : host_pinned(f_ext) && host_pinned(r) && host_pinned(v));
+    if (direct) {
         const long long step = s->step;
-        // the flag may hold this step index from before a lbp_set_step_index or a
-        // checkpoint load; the previous call's kernel has finished writing it
-        __atomic_store_n(s->h_xflag, -1ll, __ATOMIC_RELEASE);
-        TRY(step_once(s, whole));
-        TRY(wait_exchange_flag(s, step));
+        TRY(exchange_step(s, f_ext, r, v, on_device));
+        // host buffers: return once f_ext has been consumed and r, v are on the
+        // host; the step's lattice pass may still run, and later work on s0
+        // follows it.  Device buffers: stream-ordered like any other step.
+        if (!on_device) TRY(wait_exchange_flag(s, step));
         return leave(s);
     }
     const cudaMemcpyKind in = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const cudaMemcpyKind out = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     TRY(exchange_in(s, f_ext, in));
-    TRY(step_once(s));
+    bool follows = false;
+    TRY(step_once(s, follows));
     TRY(exchange_out(s, r, v, out, s->s0));
     if (!on_device) CK(cudaStreamSynchronize(s->s0));
     return leave(s);
@@ -1038,7 +965,6 @@ lbp_status lbp_set_step_index(lbp_sim *s, int64_t step) {
     CK(cudaStreamSynchronize(s->s0));
     s->step = step;
     s->vacf_lag = -1;
-    drop_graphs(s);
     return leave(s);
 }
 
@@ -1059,7 +985,6 @@ lbp_status lbp_vacf_configure_ex(lbp_sim *s, int max_lag, int per_particle) {
     TRY(enter(s));
     TRY(join_vacf(s));
     CK(cudaStreamSynchronize(s->s0));
-    drop_graphs(s);
     s->vacf_lag = -1;
     void **bufs[] = {(void **)&s->ring,   (void **)&s->ring16,   (void **)&s->vacf_sum, (void **)&s->vacf_cnt,
                      (void **)&s->vacf_part, (void **)&s->corr_g, (void **)&s->corr_h,
@@ -1191,7 +1116,6 @@ lbp_status lbp_set_body_force(lbp_sim *s, int replica, const double *g) {
             s->reps[r].gy = (float)g[1];
             s->reps[r].gz = (float)g[2];
         }
-    drop_graphs(s);  // the graphs hold the replica table by value
     return leave(s);
 }
 
@@ -1207,7 +1131,6 @@ lbp_status lbp_set_block_shape(lbp_sim *s, int rows, int variant) {
     CK(cudaStreamSynchronize(s->s0));
     s->rows = variant == 2 ? 1 : rows;
     s->variant = variant;
-    drop_graphs(s);
     return leave(s);
 }
 
@@ -1283,7 +1206,6 @@ lbp_status lbp_autotune(lbp_sim *s, int launches, int *rows, int *variant, doubl
         if (t[k] > 0 && (best < 0 || t[k] < t[best])) best = k;
     s->variant = cand_v[best];
     s->rows = cand_r[best];
-    drop_graphs(s);
     if (rows) *rows = s->rows;
     if (variant) *variant = s->variant;
     if (ms)
@@ -1331,7 +1253,8 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
                                    sizeof(double) * 3 * s->cap, cudaMemcpyDeviceToDevice, s->s0));
             }
         }
-        TRY(step_once(s));
+        bool follows = false;  // copies were queued since the last step
+        TRY(step_once(s, follows));
         if (vt) CK(launch_soa_to_aos(s->v, vt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
         if (rt) CK(launch_soa_to_aos(s->r, rt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
     }
@@ -1708,7 +1631,6 @@ lbp_status lbp_checkpoint_load(lbp_sim *s, const void *buf, int on_device) {
     CK(cudaStreamSynchronize(s->s0));
     s->step = h[5];
     s->vacf_lag = -1;  // as lbp_set_step_index: the VACF restarts from a new configure
-    drop_graphs(s);
     return leave(s);
 }
 
@@ -1718,7 +1640,6 @@ lbp_status lbp_set_wait_bound(lbp_sim *s, int64_t cycles) {
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
     s->wait_cycles = cycles == 0 ? DEFAULT_WAIT_CYCLES : (long long)cycles;
-    drop_graphs(s);  // the graphs hold the bound as a kernel parameter
     return leave(s);
 }
 
@@ -1727,7 +1648,6 @@ lbp_status lbp_set_wait_probe(lbp_sim *s, int enable) {
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
     s->wait_probe = enable ? 1 : 0;
-    drop_graphs(s);  // the graphs hold the probe flag as a kernel parameter
     return leave(s);
 }
 
@@ -1744,7 +1664,6 @@ lbp_status lbp_budget_track(lbp_sim *s, int enable) {
         cudaFree(s->inj);
         s->inj = nullptr;
     }
-    drop_graphs(s);  // the particle kernel's arguments change
     return leave(s);
 }
 
@@ -1781,8 +1700,7 @@ lbp_status lbp_budget(lbp_sim *s, double *out) {
 
 lbp_status lbp_set_use_graphs(lbp_sim *s, int enable) {
     CHECK_SIM(s);
-    s->use_graphs = enable ? 1 : 0;
-    if (!enable) drop_graphs(s);
+    s->chain = enable ? 1 : 0;
     return LBP_OK;
 }
 

@@ -47,7 +47,7 @@ __host__ __device__ constexpr float wgtf(int a) {
 //          |g/w| up to 64 still fits.
 constexpr float F16_SCALE = 1024.f;
 
-// load/store: the deviation g.  cload/cstore (and cload_shared): the values
+// load/store: the deviation g (gather: the same load through L2).  cload/cstore (and cload_shared): the values
 // the lattice kernels' collision works on (collide_st): g itself for F32 and
 // BF16; for F16 the stored variable h = g F16_SCALE / w_a, on which the
 // collision is written directly (collide_values_scaled), so the lattice pass
@@ -56,9 +56,11 @@ struct StoreF32 {
     using T = float;
     static constexpr bool SCALED = false;
     static __device__ __forceinline__ float load(const T *p, int) { return __ldg(p); }
+    static __device__ __forceinline__ float gather(const T *p, int) { return __ldcg(p); }
     static __device__ __forceinline__ float load_shared(const T *p, int) { return *p; }
     static __device__ __forceinline__ void store(T *p, int, float v) { *p = v; }
-    static __device__ __forceinline__ float cload(const T *p, int a) { return load(p, a); }
+    // through L2: a chained step reads populations before its launch dependency resolves
+    static __device__ __forceinline__ float cload(const T *p, int) { return __ldcg(p); }
     static __device__ __forceinline__ float cload_shared(const T *p, int a) { return load_shared(p, a); }
     static __device__ __forceinline__ void cstore(T *p, int a, float v) { store(p, a, v); }
 };
@@ -66,9 +68,10 @@ struct StoreBF16 {
     using T = __nv_bfloat16;
     static constexpr bool SCALED = false;
     static __device__ __forceinline__ float load(const T *p, int) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ float gather(const T *p, int) { return __bfloat162float(__ldcg(p)); }
     static __device__ __forceinline__ float load_shared(const T *p, int) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store(T *p, int, float v) { *p = __float2bfloat16_rn(v); }
-    static __device__ __forceinline__ float cload(const T *p, int a) { return load(p, a); }
+    static __device__ __forceinline__ float cload(const T *p, int) { return __bfloat162float(__ldcg(p)); }
     static __device__ __forceinline__ float cload_shared(const T *p, int a) { return load_shared(p, a); }
     static __device__ __forceinline__ void cstore(T *p, int a, float v) { store(p, a, v); }
 };
@@ -78,13 +81,16 @@ struct StoreF16 {
     static __device__ __forceinline__ float load(const T *p, int a) {
         return __half2float(__ldg(p)) * (wgtf(a) * (1.f / F16_SCALE));
     }
+    static __device__ __forceinline__ float gather(const T *p, int a) {
+        return __half2float(__ldcg(p)) * (wgtf(a) * (1.f / F16_SCALE));
+    }
     static __device__ __forceinline__ float load_shared(const T *p, int a) {
         return __half2float(*p) * (wgtf(a) * (1.f / F16_SCALE));
     }
     static __device__ __forceinline__ void store(T *p, int a, float v) {
         *p = __float2half_rn(v * (F16_SCALE / wgtf(a)));
     }
-    static __device__ __forceinline__ float cload(const T *p, int) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float cload(const T *p, int) { return __half2float(__ldcg(p)); }
     static __device__ __forceinline__ float cload_shared(const T *p, int) { return __half2float(*p); }
     static __device__ __forceinline__ void cstore(T *p, int, float v) { *p = __float2half_rn(v); }
 };
@@ -208,11 +214,26 @@ __device__ __forceinline__ void collide_st(const float g[Q], float omega, float 
 }
 
 // Programmatic dependent launch.  A step's lattice pass is launched as the
-// programmatic dependent of the step's particle kernel: the particle kernel
-// lets it start early, and the lattice kernel issues its population loads
-// (which do not depend on the particle kernel) before it waits for the
-// particle kernel to complete and its writes (force records, overflow
-// accumulator) to be visible.  Both are no-ops for ordinary launches.
+// programmatic dependent of the step's particle kernel, and within one lbp_step
+// call the next particle kernel as that of the lattice pass (one node per
+// thread), so that each is resident, with its independent loads under way, when
+// the one before it ends.  What is ordered how:
+//   * the particle kernel waits (grid_dependency_wait: the lattice pass before
+//     it is complete and visible) before it reads populations or the step
+//     index or writes anything, and lets its dependent start only after that;
+//     before, it reads only particle state, which its own predecessor wrote
+//     two launches earlier;
+//   * the lattice pass reads the populations before its wait: they are complete,
+//     because every particle block had waited for them when it let this grid
+//     start.  Its block 0 always waits, before it lets the next particle
+//     kernel start, so a lattice pass never ends before its particle kernel;
+//   * what is read ahead of a wait, or was written by a kernel of the same
+//     chain, is loaded through L2 (__ldcg): no launch boundary between the
+//     chain's kernels is relied on to invalidate L1.
+// The wait and the trigger are no-ops for ordinary launches.  us per step,
+// before (a graph replay per step) and after: 14.35 -> 10.68 (32^3, one
+// particle), 18.4 -> 14.5 (64^3, 256), 54.7 -> 51.0 (128^3, 2000), 344.5 -> 340.3
+// (256^3, 16384).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -458,16 +479,7 @@ struct Sim {
     double *stage = nullptr;
     size_t stage_bytes = 0;
 
-    // graphs
-    int use_graphs = 1;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // one step, by buffer parity
-    // lbp_step_exchange with page-locked host or device buffers: the step whose
-    // particle kernel does the I/O, by parity, with the buffer addresses, their
-    // side and the particle count it was captured for
-    cudaGraphExec_t xgraph[2] = {nullptr, nullptr};
-    const void *xkey[2][3] = {};
-    int xkey_np[2] = {0, 0};
-    int xkey_dev[2] = {0, 0};
+    int chain = 1;  // launch the steps of one call as a chain of programmatic dependents
     int vacf_pending = 0;  // a VACF block runs on s1 (ev_join marks its end)
 
     // kernel timing
@@ -478,6 +490,24 @@ struct Sim {
     double timed_ms = 0.0;
     int64_t timed_launches = 0;
 };
+
+// Launch `kern` on `st`; with `pdl` as the programmatic dependent of the
+// kernel launched before it on that stream (see grid_dependency_wait).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_k(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
+                     const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 
 // ------------------------------------------------------------ launchers
 // lbm_kernels.cu
@@ -493,6 +523,7 @@ cudaError_t launch_stream_collide_forced_cfg(Sim &s, const void *src, void *dst,
 void default_shape(const Sim &s, int &rows, int &variant);  // before lbp_autotune
 bool pair_kernel_ok(const Sim &s);  // 2-byte storage and every box with even nx
 bool variant_ok(const Sim &s, int variant);
+bool lattice_chains(const Sim &s);  // the handle's lattice kernel reads ahead through L2
 // pdl: launched right after the step's particle kernel on `st`, as its
 // programmatic dependent
 cudaError_t launch_stream_collide_forced(Sim &s, const void *src, void *dst, int parity,
@@ -516,7 +547,10 @@ struct ParticleIO {
     double *r_out, *v_out;
     bool signal;
 };
-cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io = nullptr);
+// chained: launched right after the previous step's lattice pass on `st`, as its
+// programmatic dependent
+cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io = nullptr,
+                             bool chained = false);
 bool particles_fit_per_corner(const Sim &s);  // the fit of Eq. 8 one lane per corner (few particles)
 cudaError_t launch_aos_to_soa(const double *aos, double *soa, int n, int ld, int offset,
                               cudaStream_t st);

@@ -184,19 +184,13 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
     __shared__ int s_eok[FIT8 ? PB : 1];
     const int t = threadIdx.x, lane = t & 31;
     const int i0 = blockIdx.x * PB;
-    const long long step = *A.d_step;
-    // the step's lattice pass may launch now: it waits for this grid's
-    // completion before it reads anything this kernel writes (or bumps the step)
-    grid_dependents_launch();
     const int cap = A.cap;
-    if ((A.ring || A.ring16) && blockIdx.x == 0 && t == 0) {
-        const long long m = step - A.d_vacf[0];
-        if (m >= 0) A.d_vacf[2] = m + 1;
-    }
 
     // ---- cell of each particle (warp 0): base = floor(r), q = r - base (exact).
     // Warp 0 also loads all the particle state phase B needs now, so that its
-    // loads overlap this step's other memory round trips.
+    // loads overlap this step's other memory round trips -- in a chained launch,
+    // the previous lattice pass (positions, velocities and forces were written
+    // before that pass, and are read through L2).
     const int ip = i0 + lane;
     double r0 = 0.0, r1 = 0.0, r2 = 0.0, q0 = 0.0, q1 = 0.0, q2 = 0.0;
     double V0 = 0.0, V1 = 0.0, V2 = 0.0, gam = 0.0, Rd = 0.0;
@@ -211,19 +205,19 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
                 A.fext[k * cap + ip] = f;  // kept for the steps that follow
             }
         } else {
-            s_fe[0][lane] = A.fext[ip];
-            s_fe[1][lane] = A.fext[cap + ip];
-            s_fe[2][lane] = A.fext[2 * cap + ip];
+            s_fe[0][lane] = __ldcg(A.fext + ip);
+            s_fe[1][lane] = __ldcg(A.fext + cap + ip);
+            s_fe[2][lane] = __ldcg(A.fext + 2 * cap + ip);
         }
         s_pin[lane] = A.pinned[ip];
     }
     if (t < PB && ip < A.np) {
-        r0 = A.r[ip];
-        r1 = A.r[cap + ip];
-        r2 = A.r[2 * cap + ip];
-        V0 = A.v[ip];
-        V1 = A.v[cap + ip];
-        V2 = A.v[2 * cap + ip];
+        r0 = __ldcg(A.r + ip);
+        r1 = __ldcg(A.r + cap + ip);
+        r2 = __ldcg(A.r + 2 * cap + ip);
+        V0 = __ldcg(A.v + ip);
+        V1 = __ldcg(A.v + cap + ip);
+        V2 = __ldcg(A.v + 2 * cap + ip);
         gam = A.gamma[ip];
         Rd = A.radius[ip];
         s_rep[lane] = MAXR == 1 ? 0 : A.prep[ip];
@@ -243,6 +237,16 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
             s_V[lane][1] = V1;
             s_V[lane][2] = V2;
         }
+    }
+    // the previous lattice pass is complete: populations, step index, records
+    grid_dependency_wait();
+    const long long step = __ldcg(A.d_step);
+    // the step's lattice pass may launch now: it waits for this grid's
+    // completion before it reads anything this kernel writes (or bumps the step)
+    grid_dependents_launch();
+    if ((A.ring || A.ring16) && blockIdx.x == 0 && t == 0) {
+        const long long m = step - A.d_vacf[0];
+        if (m >= 0) A.d_vacf[2] = m + 1;
     }
     __syncthreads();
 
@@ -265,7 +269,7 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
         for (int a = 1; a < Q; ++a) {
             const long long src = (long long)a * A.P + rj.node_off +
                                   ((long long)zs[ez(a) + 1] * ny + ys[ey(a) + 1]) * nx + xs[ex(a) + 1];
-            const float gv = St::load(G + src, a);
+            const float gv = St::gather(G + src, a);
             if (ex(a)) sx += ex(a) > 0 ? gv : -gv;
             if (ey(a)) sy += ey(a) > 0 ? gv : -gv;
             if (ez(a)) sz += ez(a) > 0 ? gv : -gv;
@@ -587,12 +591,13 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
 }
 
 template <int MAXR, int PB, bool FIT8>
-static void launch_particles_pb(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st) {
+static cudaError_t launch_particles_pb(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st,
+                                       bool chained) {
     const unsigned grid = (unsigned)((s.np + PB - 1) / PB);
     switch (s.precision) {
-        case LBP_BF16: k_particles<StoreBF16, MAXR, PB, FIT8><<<grid, 8 * PB, 0, st>>>(A, t); break;
-        case LBP_F16: k_particles<StoreF16, MAXR, PB, FIT8><<<grid, 8 * PB, 0, st>>>(A, t); break;
-        default: k_particles<StoreF32, MAXR, PB, FIT8><<<grid, 8 * PB, 0, st>>>(A, t); break;
+        case LBP_BF16: return launch_k(k_particles<StoreBF16, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
+        case LBP_F16: return launch_k(k_particles<StoreF16, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
+        default: return launch_k(k_particles<StoreF32, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
     }
 }
 
@@ -602,14 +607,14 @@ static void launch_particles_pb(const Sim &s, const ParticleArgs &A, const RepTa
 bool particles_fit_per_corner(const Sim &s) { return s.np < 48 * (s.num_sms > 0 ? s.num_sms : 1); }
 
 template <int MAXR>
-static void launch_particles_t(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st) {
-    if (particles_fit_per_corner(s))
-        launch_particles_pb<MAXR, PB_NARROW, true>(s, A, t, st);
-    else
-        launch_particles_pb<MAXR, PB_WIDE, false>(s, A, t, st);
+static cudaError_t launch_particles_t(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st,
+                                      bool chained) {
+    if (particles_fit_per_corner(s)) return launch_particles_pb<MAXR, PB_NARROW, true>(s, A, t, st, chained);
+    return launch_particles_pb<MAXR, PB_WIDE, false>(s, A, t, st, chained);
 }
 
-cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io) {
+cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io,
+                             bool chained) {
     if (s.np == 0) return cudaSuccess;
     ParticleArgs A;
     A.g = src;
@@ -654,15 +659,14 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
         t.item_off[0] = 0;
         t.item_off[1] = 0;
         t.rep[0] = s.reps[0];
-        launch_particles_t(s, A, t, st);
+        return launch_particles_t(s, A, t, st, chained);
     } else {
         RepTable<MAX_BATCH> t;  // kernel parameter
         t.nrep = s.nrep;
         for (int r = 0; r <= s.nrep; ++r) t.item_off[r] = 0;
         for (int r = 0; r < s.nrep; ++r) t.rep[r] = s.reps[r];
-        launch_particles_t(s, A, t, st);
+        return launch_particles_t(s, A, t, st, chained);
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

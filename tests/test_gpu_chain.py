@@ -1,0 +1,59 @@
+"""The steps of one call, launched as a chain, against the same steps one call each: bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_1909_13412_gb300 import lbp  # noqa: E402
+from paper_1909_13412_gb300 import workloads as wl  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def run(boxes, counts, precision, mode, calls, shape, chain=True, lag=-1):
+    h = lbp.lbp_create_batch([(*b, 0.8) for b in boxes], precision=precision)
+    if shape is not None:
+        lbp.lbp_set_block_shape(h, *shape)
+    lbp.lbp_set_use_graphs(h, chain)
+    for k, ((nx, ny, nz), n) in enumerate(zip(boxes, counts)):
+        if n:
+            ps = wl.uniform_particles(n, (nz, ny, nx), 10.0, 0.5, 0.26, 1e-3, 5 + k, 6 + k)
+            lbp.lbp_particles_add_to(h, k, ps.r, ps.V * 30, ps.M, ps.gamma, ps.R)
+    lbp.lbp_particles_set_params(h, kT=1e-3, seed=3, mode=mode)
+    if lag >= 0:
+        lbp.lbp_vacf_configure(h, lag)
+    for n in calls:
+        lbp.lbp_step(h, n)
+    n = sum(counts)
+    out = [np.empty(15 * h.N)] + [np.empty((n, 3)) for _ in range(4)]
+    lbp.lbp_read_populations(h, out[0])
+    lbp.lbp_particles_read(h, *out[1:])
+    if lag >= 0:
+        out += [np.empty(lag + 1), np.empty(lag + 1, np.int64)]
+        lbp.lbp_vacf_read(h, *out[-2:])
+    lbp.lbp_check(h)
+    lbp.lbp_destroy(h)
+    return out
+
+
+@pytest.mark.parametrize("boxes,counts", [
+    ([(32, 32, 32)], [1]),              # a few marked rows
+    ([(3, 5, 131)], [40]),              # corners that wrap in every direction, records that overflow
+    ([(260, 9, 8)], [300]),             # three segments a row, most rows marked
+    ([(96, 64, 64)], [9000]),           # one thread per particle
+    ([(64, 20, 20), (17, 9, 30), (130, 8, 8)], [2, 0, 30])])
+@pytest.mark.parametrize("precision,shape", [
+    (lbp.LBP_F32, None), (lbp.LBP_F32, (1, 0)), (lbp.LBP_F32, (4, 0)), (lbp.LBP_BF16, (2, 0)), (lbp.LBP_F16, None),
+    (lbp.LBP_BF16, None)])
+def test_steps_of_one_call_equal_single_calls(boxes, counts, precision, shape):
+    want = run(boxes, counts, precision, lbp.LBP_STOKESLET, [1] * 40, shape, chain=False)
+    for calls in ([40], [7, 33]):
+        got = run(boxes, counts, precision, lbp.LBP_STOKESLET, calls, shape)
+        assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("mode", [lbp.LBP_POINTWISE, lbp.LBP_BROWNIAN])
+def test_chained_modes_and_correlator_blocks(mode):
+    args = ([(40, 36, 34)], [50], lbp.LBP_F32, mode)
+    want = run(*args, [1] * 150, None, chain=False, lag=30)
+    got = run(*args, [150], None, lag=30)
+    assert all(np.array_equal(a, b) for a, b in zip(got, want))
