@@ -148,8 +148,8 @@ __device__ __forceinline__ void record_sum(unsigned long long rw, int cnt, int x
 // ---------------------------------------------------------------------------
 template <int BX, typename St, int R, int MAXR>
 __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
-    Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *__restrict__ rec_cur,
-    unsigned long long *rec_prev, unsigned long long *fq, long long Ntot, long long *bump, int *err) {
+    Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *rec_cur, unsigned long long *rec_prev,
+    unsigned long long *fq, long long Ntot, long long *bump, int *err, const Marks mk) {
     static_assert(BX == SEG, "one block per force-record segment");
     const int r = find_block_rep(rt, blockIdx.x);
     const Rep &rp = rt.rep[r];
@@ -172,26 +172,31 @@ __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
     NodeIdx n[R];
     float g[R][Q];
     unsigned long long rw[R];
-    bool bad = false;
+    bool bad = false, forced[R];
 #pragma unroll
     for (int h = 0; h < R; ++h) {
         const unsigned row = grp * R + h < nrows ? grp * R + h : nrows - 1;
         n[h] = node_index(x, row, nx, ny, nz, rp.dny);
         n[h].d += base;
+        forced[h] = mk.epoch == 0 || __ldcg(mk.seg + seg0 + (size_t)row * nchunks + chunk) == mk.epoch;
 #pragma unroll
         for (int a = 0; a < Q; ++a)
             g[h][a] = St::cload(pl.s[a] + (n[h].d + n[h].ox[ex(a) + 1] + n[h].oy[ey(a) + 1] +
                                           n[h].oz[ez(a) + 1]), a);
     }
-    // the loads above do not depend on this step's particle kernel; what follows does
-    // (a no-op unless launched as its programmatic dependent)
-    grid_dependency_wait();
-    grid_dependents_launch();
+    // the loads above do not depend on this step's particle kernel; the records do
+    // (the wait is a no-op unless launched as its programmatic dependent)
+    bool wait = blockIdx.x == 0;
+#pragma unroll
+    for (int h = 0; h < R; ++h) wait = wait || forced[h];
+    if (wait) grid_dependency_wait();
+    if (mk.release) grid_dependents_launch();
     if (blockIdx.x == 0 && threadIdx.x == 0) *bump += 1;
 #pragma unroll
     for (int h = 0; h < R; ++h) {
         const unsigned row = grp * R + h < nrows ? grp * R + h : nrows - 1;
-        rw[h] = __ldcg(rec_cur + (seg0 + (size_t)row * nchunks + chunk) * REC_WORDS + lane);
+        rw[h] = 0ull;
+        if (forced[h]) rw[h] = __ldcg(rec_cur + (seg0 + (size_t)row * nchunks + chunk) * REC_WORDS + lane);
     }
 #pragma unroll
     for (int h = 0; h < R; ++h) {
@@ -663,6 +668,20 @@ bool staged_kernel_ok(const Sim &s) {
 // adjacent warps share (0.172 against 0.187 ms for BF16 at 256^3 without).
 bool lattice_chains(const Sim &s) { return s.variant == 0; }
 
+// Marks let the segments without forces collide beside the particle kernel.
+// That pays once the pass has more blocks than are resident at a time (eight
+// per SM): below, all blocks already wait with their loads done, and the
+// particle kernel only loses issue slots to them (11.1 -> 11.3 us at 32^3).
+// The kernels with several nodes per thread do without: with the conditional
+// wait the four-node kernel measured 0.194 against 0.172 ms (BF16, 256^3).
+bool lattice_marks(const Sim &s) {
+    if (!lattice_chains(s) || s.np == 0) return false;
+    long long blocks = 0;
+    for (int r = 0; r < s.nrep; ++r)
+        blocks += ((long long)s.reps[r].ny * s.reps[r].nz + s.rows - 1) / s.rows * s.reps[r].nchunks;
+    return blocks > 8ll * s.num_sms;
+}
+
 // Replica table of the staged kernel: items of whole rows (Rep::pad = rows per item).
 template <int MAXR>
 static RepTable<MAXR> rep_table_staged(const Sim &s) {
@@ -694,7 +713,7 @@ bool variant_ok(const Sim &s, int variant) {
 template <bool FORCED>
 static cudaError_t launch_sc(Sim &s, const void *src, void *dst, const unsigned long long *rec_cur,
                              unsigned long long *rec_prev, long long *bump, int rows, int variant,
-                             cudaStream_t st, bool pdl = false) {
+                             cudaStream_t st, bool pdl = false, unsigned epoch = 0) {
     constexpr int BX = SC_BX;
     if (!variant_ok(s, variant)) variant = 0;
     if (variant == 2) {
@@ -710,6 +729,7 @@ static cudaError_t launch_sc(Sim &s, const void *src, void *dst, const unsigned 
         });
     }
     const bool use_pair = variant == 1, use_quad = variant == 3;
+    const Marks mk{s.marks[epoch & 1], epoch, particles_start_early(s)};
     return by_storage(s, [&](auto tag) {
         using St = decltype(tag);
         return by_rows(rows, [&](auto rc) {
@@ -728,7 +748,7 @@ static cudaError_t launch_sc(Sim &s, const void *src, void *dst, const unsigned 
                 }
                 if constexpr (FORCED)
                     return launch_k(k_stream_collide_forced<BX, St, R, MAXR>, grid, BX, 0, st, pdl,
-                                    planes_of<St>(s, src, dst), rt, rec_cur, rec_prev, s.fq, s.N, bump, s.d_err);
+                                    planes_of<St>(s, src, dst), rt, rec_cur, rec_prev, s.fq, s.N, bump, s.d_err, mk);
                 else
                     k_stream_collide<BX, St, R, MAXR><<<grid, BX, 0, st>>>(planes_of<St>(s, src, dst), rt, bump,
                                                                            s.d_err);
@@ -755,8 +775,8 @@ cudaError_t launch_stream_collide(Sim &s, const void *src, void *dst, cudaStream
 }
 
 cudaError_t launch_stream_collide_forced(Sim &s, const void *src, void *dst, int parity,
-                                         cudaStream_t st, bool pdl) {
-    return launch_sc<true>(s, src, dst, s.rec[parity], s.rec[parity ^ 1], s.d_step, s.rows, s.variant, st, pdl);
+                                         cudaStream_t st, bool pdl, unsigned epoch) {
+    return launch_sc<true>(s, src, dst, s.rec[parity], s.rec[parity ^ 1], s.d_step, s.rows, s.variant, st, pdl, epoch);
 }
 
 // ---------------------------------------------------------------------------

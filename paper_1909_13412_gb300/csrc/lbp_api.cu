@@ -131,19 +131,20 @@ double nu_of(double tau) { return (tau - 0.5) / 3.0; }
 // writes the positions and velocities itself, and for host buffers raises the
 // step's completion flag.  `chained`: the previous launch on s0 was the lattice
 // pass of the step before, of which the particle kernel becomes the
-// programmatic dependent.
-lbp_status enqueue_step(lbp_sim *s, bool timed, bool chained, const ParticleIO *io) {
+// programmatic dependent.  `epoch`: the step before marked this step's
+// segments with it (0: it did not); `next`: mark the next step's (0: do not).
+lbp_status enqueue_step(lbp_sim *s, bool timed, bool chained, unsigned epoch, unsigned next, const ParticleIO *io) {
     Range range("lbp step: particles + lattice pass");
     const void *src = s->f[s->cur];
     void *dst = s->f[s->cur ^ 1];
     const int parity = s->cur;
-    if (s->np > 0) CK(launch_particles(*s, src, parity, s->s0, io, chained));
+    if (s->np > 0) CK(launch_particles(*s, src, parity, s->s0, io, chained, next));
     if (timed) CK(cudaEventRecord(s->tev[2 * s->ntimed], s->s0));
     // the lattice pass as the programmatic dependent of the particle kernel
     // (its population loads overlap the particle kernel's tail); not when
     // events around it time the lattice kernel alone
     if (s->np > 0)
-        CK(launch_stream_collide_forced(*s, src, dst, parity, s->s0, !timed));
+        CK(launch_stream_collide_forced(*s, src, dst, parity, s->s0, !timed, epoch));
     else
         CK(launch_stream_collide(*s, src, dst, s->s0));
     if (timed) {
@@ -189,10 +190,16 @@ lbp_status fold_timing(lbp_sim *s) {
     return LBP_OK;
 }
 
-// one time step on s0.  `follows`: the last thing queued on s0 is the lattice
-// pass of the step before (within one call), so the two can be chained; on
-// return it says the same for the next step.
-lbp_status step_once(lbp_sim *s, bool &follows, const ParticleIO *io = nullptr) {
+// What the steps of one call hand to one another.  Nothing is kept from call to
+// call: a first step relies neither on what was queued before it nor on marks.
+struct Chain {
+    int64_t left;          // steps of the call not yet queued
+    bool follows = false;  // the last thing on s0 is the lattice pass of the step before
+    unsigned epoch = 0;    // the step before marked this step's segments with this epoch
+};
+
+// one time step on s0
+lbp_status step_once(lbp_sim *s, Chain &c, const ParticleIO *io = nullptr) {
     // the VACF correlator runs when the step completes a block of B samples
     const int B = vacf_block_samples();
     bool due = false;
@@ -205,8 +212,11 @@ lbp_status step_once(lbp_sim *s, bool &follows, const ParticleIO *io = nullptr) 
     }
     const bool timed = s->timing != 0;
     if (timed && s->ntimed == lbp::Sim::MAX_TIMED) TRY(fold_timing(s));
-    TRY(enqueue_step(s, timed, follows && !timed && s->chain && lattice_chains(*s), io));
-    follows = !due;
+    const unsigned next = c.left > 1 && s->chain && lattice_marks(*s) ? ++s->epoch : 0;  // 0 also when it wraps
+    TRY(enqueue_step(s, timed, c.follows && !timed && s->chain && lattice_chains(*s), c.epoch, next, io));
+    c.epoch = next;
+    c.follows = !due;
+    c.left -= 1;
     if (due) TRY(fork_vacf(s));
     s->cur ^= 1;
     s->step += 1;
@@ -268,8 +278,8 @@ lbp_status exchange_step(lbp_sim *s, const double *f_ext, double *r, double *v, 
         __atomic_store_n(s->h_xflag, -1ll, __ATOMIC_RELEASE);
     }
     const ParticleIO io{f_dev, r_dev, v_dev, !on_device};
-    bool follows = false;
-    return step_once(s, follows, &io);
+    Chain c{1};
+    return step_once(s, c, &io);
 }
 
 // Wait until the particle kernel of step `step` has written the positions and
@@ -479,7 +489,7 @@ lbp_status lbp_destroy(lbp_sim *s) {
     free_tape(s);
     void *bufs[] = {s->f[0], s->f[1], s->d_step, s->d_err, s->r, s->v, s->fh, s->fr, s->fext, s->xbuf,
                     s->mass, s->inv_mass, s->gamma, s->radius, s->sig, s->pinned, s->prep, s->fq, s->rec[0],
-                    s->rec[1], s->ring,
+                    s->rec[1], s->marks[0], s->marks[1], s->ring,
                     s->d_vacf, s->vacf_sum, s->vacf_cnt, s->vacf_part, s->stage, s->inj, s->budget_part,
                     s->corr_g, s->corr_h, s->corr_w, s->msd_state, s->msd_sum, s->ring16, s->d_xticket};
     for (void *b : bufs)
@@ -690,6 +700,8 @@ lbp_status lbp_particles_add_to(lbp_sim *s, int replica, int n, const double *r,
             for (int q = 0; q < 2; ++q) {
                 TRY(dalloc(&s->rec[q], (size_t)s->nseg * REC_WORDS));
                 CK(cudaMemset(s->rec[q], 0, sizeof(unsigned long long) * (size_t)s->nseg * REC_WORDS));
+                TRY(dalloc(&s->marks[q], (size_t)s->nseg));
+                CK(cudaMemset(s->marks[q], 0, sizeof(unsigned) * (size_t)s->nseg));
             }
         }
         s->cap = cap;
@@ -911,8 +923,8 @@ lbp_status lbp_step(lbp_sim *s, int64_t nsteps) {
     if (nsteps < 0) return fail(LBP_EINVAL, "lbp_step: nsteps < 0");
     if (nsteps == 0) return LBP_OK;
     TRY(enter(s));
-    bool follows = false;
-    for (int64_t n = 0; n < nsteps; ++n) TRY(step_once(s, follows));
+    Chain c{nsteps};
+    for (int64_t n = 0; n < nsteps; ++n) TRY(step_once(s, c));
     return leave(s);
 }
 
@@ -948,8 +960,8 @@ lbp_status lbp_step_exchange(lbp_sim *s, const double *f_ext, double *r, double 
     const cudaMemcpyKind in = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const cudaMemcpyKind out = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     TRY(exchange_in(s, f_ext, in));
-    bool follows = false;
-    TRY(step_once(s, follows));
+    Chain c{1};
+    TRY(step_once(s, c));
     TRY(exchange_out(s, r, v, out, s->s0));
     if (!on_device) CK(cudaStreamSynchronize(s->s0));
     return leave(s);
@@ -1241,6 +1253,7 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     tp.C = checkpoint_every;
     tp.np = s->np;
     tp.nck = nck;
+    Chain c{nsteps};
     for (int64_t n = 0; n < nsteps; ++n) {
         if (n % checkpoint_every == 0) {
             const int64_t k = n / checkpoint_every;
@@ -1253,8 +1266,8 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
                                    sizeof(double) * 3 * s->cap, cudaMemcpyDeviceToDevice, s->s0));
             }
         }
-        bool follows = false;  // copies were queued since the last step
-        TRY(step_once(s, follows));
+        c.follows = false;  // copies were queued since the last step
+        TRY(step_once(s, c));
         if (vt) CK(launch_soa_to_aos(s->v, vt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
         if (rt) CK(launch_soa_to_aos(s->r, rt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
     }

@@ -72,6 +72,8 @@ struct ParticleArgs {
     int mode, exclude_inside;
     unsigned long long *rec; // force records of this step's parity
     unsigned long long *fq;  // [3][N] fixed-point overflow accumulator
+    unsigned *marks;         // next step's marks (Marks), or null
+    unsigned mark_epoch;
     float *ring;        // per-particle VACF ring (FP32), or null
     __half *ring16;     // ensemble VACF/MSD ring (fp16 hi/lo planes), or null
     int ring_ld, ring_dup;
@@ -173,6 +175,7 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
     __shared__ long long s_fix[PB][3];
     __shared__ long long s_frac[PB][3];
     __shared__ int s_spread[PB];
+    __shared__ int s_next[PB][3];  // cell after the update
     // state read only by the Langevin update, staged by warp 1 so that warp 0
     // (the FP64 fit) carries fewer registers across the gather
     __shared__ double s_fe[3][PB];
@@ -463,6 +466,7 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
                 A.r[k * cap + i] = rn;
                 rw = rn;
             }
+            if (A.marks) s_next[lane][k] = (int)floor(rw);
             if (FIT8) {  // few particles: straight from the update's registers
                 if (A.r_out) A.r_out[3 * (size_t)i + k] = rw;
                 if (A.v_out) A.v_out[3 * (size_t)i + k] = Vn[k];
@@ -573,6 +577,13 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
         }
     }
 
+    // mark the row segment of corner p of the next step's cell
+    if (A.marks && ij < A.np) {
+        const int x1 = wrapi(s_next[j][0] + c0, nx), y1 = wrapi(s_next[j][1] + c1, ny),
+                  z1 = wrapi(s_next[j][2] + c2, nz);
+        A.marks[rj.seg_off + ((long long)z1 * ny + y1) * rj.nchunks + x1 / SEG] = A.mark_epoch;
+    }
+
     // the last block to finish tells the host that every position and velocity
     // is in its buffers (the lattice pass may still run)
     if (A.done_flag) {
@@ -606,6 +617,14 @@ static cudaError_t launch_particles_pb(const Sim &s, const ParticleArgs &A, cons
 // dependent chain, not the pipe, sets the time); both give the same bits.
 bool particles_fit_per_corner(const Sim &s) { return s.np < 48 * (s.num_sms > 0 ? s.num_sms : 1); }
 
+// Whether the lattice pass lets the next particle kernel start before it ends.
+// Blocks that start while the pass drains crowd onto the SMs that empty first,
+// and the FP64 pipe (16 cycles a warp instruction) serves their fits one after
+// another: 63 narrow blocks at 80^3 took 37 instead of 13 us.  So early only
+// where they cannot crowd: the wide layout (at most four blocks per SM;
+// 341.4 -> 337.5 us a step at 256^3) and a single block (23.2 -> 22.2 us at 100^3).
+bool particles_start_early(const Sim &s) { return !particles_fit_per_corner(s) || s.np <= PB_NARROW; }
+
 template <int MAXR>
 static cudaError_t launch_particles_t(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st,
                                       bool chained) {
@@ -614,7 +633,7 @@ static cudaError_t launch_particles_t(const Sim &s, const ParticleArgs &A, const
 }
 
 cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io,
-                             bool chained) {
+                             bool chained, unsigned mark_epoch) {
     if (s.np == 0) return cudaSuccess;
     ParticleArgs A;
     A.g = src;
@@ -640,6 +659,9 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
     A.exclude_inside = s.exclude_inside;
     A.fq = s.fq;
     A.rec = s.rec[parity];
+    // Eq. 6 spreads nothing: no segment of the next step waits
+    A.marks = mark_epoch && s.mode != LBP_BROWNIAN ? s.marks[mark_epoch & 1] : nullptr;
+    A.mark_epoch = mark_epoch;
     A.ring = s.vacf_lag >= 0 && s.vacf_pp ? s.ring : nullptr;
     A.ring16 = s.vacf_lag >= 0 && !s.vacf_pp ? static_cast<__half *>(s.ring16) : nullptr;
     A.ring_ld = s.ring_ld;
