@@ -303,7 +303,7 @@ lbp_status lbp_check(lbp_sim *sim);
  * no pinned particle and no body force, out[1..3] + out[4..6] - out[7..9]
  * keeps its value from when tracking began, to rounding; a uniform body force
  * g (lbp_set_body_force) adds N g per step, which the caller accounts for.
- * Tracking adds one FP64 atomic per 32 particles and component to every step;
+ * Tracking adds one FP64 atomic per 16 particles and component to every step;
  * lbp_budget_track(sim, 0) stops it.                                         */
 lbp_status lbp_budget_track(lbp_sim *sim, int enable);
 lbp_status lbp_budget(lbp_sim *sim, double *out);
@@ -332,9 +332,10 @@ lbp_status lbp_set_wait_probe(lbp_sim *sim, int enable);
  * force accumulation; the results do not depend on them), out[1] = capacity of
  * a record in shares, out[2] = number of row segments, out[3] = rows of 128
  * nodes per lattice-kernel block, out[4] = its variant (see lbp_autotune),
- * out[5] = 1 if the particle kernel fits Eq. 8 with one lane per cell corner
- * (fewer than 48 particles per SM), 0 if with one thread per particle; both
- * layouts give the same bits.  n = entries of out (up to 6).                 */
+ * out[5] = 1 with fewer than 48 particles per SM, where the particle kernel
+ * prepares the corners' geometry before the lattice pass ahead of it ends, 0
+ * from there on, where it does so while its gather is in flight; both give the
+ * same bits.  n = entries of out (up to 6).                                   */
 lbp_status lbp_diagnostics(lbp_sim *sim, int64_t *out, int n);
 
 /* Uniform body force density g = (gx, gy, gz) added on every node of box

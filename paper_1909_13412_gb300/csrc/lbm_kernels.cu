@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
 #pragma unroll
     for (int h = 0; h < R; ++h) wait = wait || forced[h];
     if (wait) grid_dependency_wait();
-    if (mk.release) grid_dependents_launch();
+    grid_dependents_launch();
     if (blockIdx.x == 0 && threadIdx.x == 0) *bump += 1;
 #pragma unroll
     for (int h = 0; h < R; ++h) {
@@ -729,7 +729,7 @@ static cudaError_t launch_sc(Sim &s, const void *src, void *dst, const unsigned 
         });
     }
     const bool use_pair = variant == 1, use_quad = variant == 3;
-    const Marks mk{s.marks[epoch & 1], epoch, particles_start_early(s)};
+    const Marks mk{s.marks[epoch & 1], epoch};
     return by_storage(s, [&](auto tag) {
         using St = decltype(tag);
         return by_rows(rows, [&](auto rc) {

@@ -462,7 +462,7 @@ lbp_status lbp_create_batch(const lbp_lattice_desc *descs, int nrep, void *strea
         st = dalloc(&buf, (size_t)storage_bytes(s->precision) * Q * s->P);
         s->f[i] = buf;
     }
-    if (st == LBP_OK) st = dalloc(&s->d_step, 1);
+    if (st == LBP_OK) st = dalloc(&s->d_step, 3);
     if (st == LBP_OK) st = dalloc(&s->d_err, 1);
     if (st == LBP_OK) st = dalloc(&s->d_vacf, 8);
 
@@ -1526,7 +1526,7 @@ lbp_status lbp_diagnostics(lbp_sim *s, int64_t *out, int n) {
     CHECK_SIM(s);
     if (n < 0 || (n > 0 && !out)) return fail(LBP_EINVAL, "lbp_diagnostics: bad output");
     CK(cudaStreamSynchronize(s->s0));
-    int64_t v[6] = {0, REC_SLOTS, s->nseg, s->rows, (int64_t)s->variant, particles_fit_per_corner(*s) ? 1 : 0};
+    int64_t v[6] = {0, REC_SLOTS, s->nseg, s->rows, (int64_t)s->variant, particles_few(*s) ? 1 : 0};
     if (s->rec[0]) {
         // shares beyond the slots of the records of the last completed step
         std::vector<unsigned long long> words((size_t)s->nseg * REC_WORDS);

@@ -290,7 +290,6 @@ constexpr int REC_F0 = 5;
 struct Marks {
     const unsigned *seg;  // [segments], the array of this epoch's parity
     unsigned epoch;       // 0: no marks, every segment waits
-    bool release;         // let the next particle kernel start before this pass ends
 };
 
 // error bits in Sim::d_err
@@ -429,7 +428,7 @@ struct Sim {
     void *f[2] = {nullptr, nullptr};   // deviation populations, 15 planes of P (storage type)
     int cur = 0;                       // f[cur] holds fhat^n
     int64_t step = 0;                  // host mirror of the step index
-    long long *d_step = nullptr;       // device step index (Philox counter)
+    long long *d_step = nullptr;       // device step index (Philox counter), and two slots of the particle kernel's
     int *d_err = nullptr;
 
     // particles, FP64 structure of arrays, 3 planes of cap for vectors
@@ -572,8 +571,7 @@ struct ParticleIO {
 // its epoch (0: do not)
 cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io = nullptr,
                              bool chained = false, unsigned mark_epoch = 0);
-bool particles_start_early(const Sim &s);     // launch them before the lattice pass before them ends
-bool particles_fit_per_corner(const Sim &s);  // the fit of Eq. 8 one lane per corner (few particles)
+bool particles_few(const Sim &s);  // the particle kernel prepares ahead of its launch dependency
 cudaError_t launch_aos_to_soa(const double *aos, double *soa, int n, int ld, int offset,
                               cudaStream_t st);
 cudaError_t launch_soa_to_aos(const double *soa, double *aos, int n, int ld, cudaStream_t st);

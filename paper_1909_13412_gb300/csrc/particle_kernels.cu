@@ -1,35 +1,56 @@
 // particle_kernels.cu -- two-way coupling kernel of liblbp (sm_103a).
 //
-// k_particles: a block of 8 PB threads serves PB particles in three phases.
-//   A. eight threads per particle (one per corner) gather u^N at the corners
-//      of the particle's cell from the stored populations (a pull, i.e. the
-//      streamed f^n of Eq. 20): 14 independent loads per thread;
-//   B. the Stokeslet flow of Eq. 8 is fitted -- by one thread per particle
-//      (PB = 32), or with few particles by its eight corner lanes (PB = 8) --
-//      and one thread per particle draws the Philox random force (Eqs. 4-5)
-//      and advances V and r (Eqs. 1-2);
-//   C. eight threads per particle append the shares of the reaction force
-//      -F_H (Eq. 9) at the corner nodes to the force records of the row
-//      segments holding those nodes; the stream-collide kernel applies them.
+// k_particles, eight lanes per particle (one per corner of its cell) and four
+// particles per warp, every step:
+//   A. gathers u^N at the corners of the particle's cell from the stored
+//      populations (a pull, i.e. the streamed f^n of Eq. 20): 14 independent
+//      loads per lane;
+//   B. fits the Stokeslet flow of Eq. 8, draws the Philox random force
+//      (Eqs. 4-5) and advances V and r (Eqs. 1-2);
+//   C. appends the shares of the reaction force -F_H (Eq. 9) at the corner
+//      nodes to the force records of the row segments holding those nodes (the
+//      stream-collide kernel applies them) and marks the segments of the next
+//      step's corners.
 //
-// Why one thread per particle in phase B: GB300 issues FP64 at 1/64 of the
-// FP32 rate, so a warp-wide FP64 instruction costs the same whether one lane
-// or 32 lanes need it.  Packing 32 particles into the warp that does the FP64
-// work divides its FP64 instruction count per particle by 32; with one
-// particle per warp the FP64 work of the fit dominated the whole time step.
-// That holds while the FP64 pipe is the limit; with a warp or two of
-// particles per SM the fit's dependent chain is, and the lane-per-corner
-// layout shortens it (see PB_WIDE / PB_NARROW below).
+// What bounds it: the FP64 pipe, and with many particles the gather.  A warp's
+// FP64 instruction takes 64 cycles whatever its active lanes and whether or not
+// it depends on the one before (measured: chains and independent FMAs alike;
+// four warps of an SM proceed beside one another), a reciprocal square root
+// seven of them, a division ten.  So a warp's time is 64 cycles times its FP64
+// instructions, and they are kept few, and out of the way:
+//   * vector operations run with one component per lane: lane p of a particle
+//     holds component comp_of(p) of r, V, F, ... (lanes 0, 2, 1 store x, y, z),
+//     so an update of three components is one instruction; the sum over the
+//     corners leaves each component in its lanes (sum_components), and the two
+//     sums of the normal equation share their additions (sum_pair);
+//   * what depends on positions alone -- the cell, the corner geometry with its
+//     reciprocal square root, the spreading fractions -- and the random force
+//     are done before the launch dependency resolves, beside the previous
+//     lattice pass (the step index comes from the previous particle kernel,
+//     step_in), or with many particles (MANY), whose gather takes longer than the
+//     end of that pass, while the gather is in flight; a warp of its own lets the
+//     lattice pass of this step launch;
+//   * comparisons and the widening of u^N are done on the bits;
+//   * every warp works by itself (no shared memory, no block barrier), so that
+//     with many particles the fits of some overlap the gathers of others.
+// About 60 FP64 instructions for four particles remain between the end of the
+// previous lattice pass and the update.  Before, after the gather one warp of a
+// block did the scalar work of 8 particles (187 instructions, few particles) or
+// one thread all of a particle's (530, many), with block barriers between the
+// phases.  us per step, before -> after: 10.8 -> 7.8 (32^3, one particle),
+// 14.4 -> 10.4 (64^3, 256), 49.6 -> 45.3 (128^3, 2000), 38.9 -> 35.2 (the same,
+// BF16), 336.4 -> 327.8 (256^3, 16384), 212.4 -> 209.0 (the same, BF16).
+// Four lanes per particle, with two corners each (85 instructions for eight
+// particles), measured slower than eight lanes from 7000 particles (73.4 against
+// 67.5 at 128^3) to 131072 (1186 against 1174 at 256^3): not kept.
 //
 // Exchange I/O (lbp_step_exchange with device buffers or page-locked host
-// buffers, seen through their device views): warp 1 reads the block's
-// external forces from the caller's [n][3] buffer and keeps them; the new
-// positions and velocities go to the caller's buffers after phase B, as one
-// contiguous span per block read back from the state arrays (PB = 32) or
-// straight from the update's registers (PB = 8).  For host buffers the last
-// block to finish then sets a completion flag in page-locked memory after a
-// system-scope fence, and the host returns without waiting for the lattice
-// pass.
+// buffers, seen through their device views): the lanes read the external forces
+// from the caller's [n][3] buffer and keep them, and write the new positions
+// and velocities to the caller's buffers (a warp's are contiguous).  For host
+// buffers the last block to finish then sets a completion flag in page-locked
+// memory after a system-scope fence, and the host returns without waiting for
+// the lattice pass.
 //
 // Precision split.  FP32: the gathered u^N (the lattice arithmetic is FP32).
 // FP64: everything after the gather -- positions, velocities, the cell and
@@ -66,7 +87,13 @@ struct ParticleArgs {
     const double *inv_mass, *gamma, *radius, *sig;
     const unsigned char *pinned;
     int cap, np;
-    const long long *d_step;
+    const long long *d_step;  // step index, bumped by the lattice pass
+    // the step index as left by the previous particle kernel of the same call, if
+    // chained, and for the next one: two slots by parity, because blocks of this
+    // grid may start after others have finished
+    const long long *step_in;
+    long long *step_out;
+    bool chained;
     unsigned long long seed;
     double sqrt3;
     int mode, exclude_inside;
@@ -93,504 +120,353 @@ struct ParticleArgs {
 
 __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// Eq. 8 in FP64, shared by both layouts of the fit below.  Every operation is
-// rounded explicitly (no contraction left to the compiler), and the eight
-// corners' terms are summed as the tree ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)),
-// which is also the order of a butterfly over eight lanes: one thread per
-// particle and one lane per corner give the same bits.
+// Component of the vectors that lane p of a particle holds, and the first lane
+// holding component k.
+__device__ __forceinline__ int comp_of(int p) { return (p & 1) ? 2 : (p >> 1) & 1; }
+__device__ __forceinline__ int lane_of(int k) { return k == 0 ? 0 : 3 - k; }
+
+// |v| < bound for bound > 0 (false for a NaN), on the bits
+__device__ __forceinline__ bool below(double v, double bound) {
+    return (__double_as_longlong(v) & 0x7fffffffffffffffll) < __double_as_longlong(bound);
+}
+
+// v < 0 (not for -0; also for a NaN with its sign set), on the bits
+__device__ __forceinline__ bool negative(double v) {
+    return (unsigned long long)__double_as_longlong(v) > 0x8000000000000000ull;
+}
+
+template <typename T>
+__device__ __forceinline__ T from_comp(T v, int k) {
+    return __shfl_sync(0xffffffffu, v, lane_of(k), 8);
+}
+
+// Sums over a particle's eight corners follow the tree
+// ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), every operation rounded explicitly.
 //
-// e^N = m/|m| of the mean relative velocity m (times 8); false if m = 0.
-__device__ __forceinline__ bool fit_direction(double m0, double m1, double m2, double &e0, double &e1,
-                                              double &e2) {
-    if (m0 == 0.0 && m1 == 0.0 && m2 == 0.0) return false;
+// The sum of (v0, v1, v2), component comp_of(p) in lane p: lanes that differ in
+// the first bit split component 2 from the others, those that differ in the
+// second 0 from 1.
+__device__ __forceinline__ double sum_components(double v0, double v1, double v2, int p) {
+    const bool odd = p & 1;
+    double a = __shfl_xor_sync(0xffffffffu, odd ? v0 : v2, 1), b = __shfl_xor_sync(0xffffffffu, v1, 1);
+    a = __dadd_rn(odd ? v2 : v0, a);
+    b = __dadd_rn(v1, b);
+    const bool one = !odd && (p & 2);
+    const double c = __shfl_xor_sync(0xffffffffu, odd || one ? a : b, 2);
+    a = __dadd_rn(one ? b : a, c);
+    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
+}
+
+// the sums of x (left in even lanes) and y (in odd lanes)
+__device__ __forceinline__ double sum_pair(double x, double y, int p) {
+    const bool odd = p & 1;
+    double a = __dadd_rn(odd ? y : x, __shfl_xor_sync(0xffffffffu, odd ? x : y, 1));
+    a = __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 2));
+    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
+}
+
+// e^N = m/|m| of the mean relative velocity m (times 8), given by its component
+// in each lane; false if m = 0
+__device__ __forceinline__ bool direction(double mk, double (&e)[3]) {
+    double m0 = from_comp(mk, 0), m1 = from_comp(mk, 1), m2 = from_comp(mk, 2);
+    const long long any = __double_as_longlong(m0) | __double_as_longlong(m1) | __double_as_longlong(m2);
     double mm = __fma_rn(m2, m2, __fma_rn(m1, m1, __dmul_rn(m0, m0)));
-    if (!(mm > 1e-280)) {
+    if (__double_as_longlong(mm) <= __double_as_longlong(1e-280)) {
         // tiny mean: rescale before the norm so that it does not underflow
         const double sc = 1.0 / fmax(fabs(m0), fmax(fabs(m1), fabs(m2)));
         m0 = __dmul_rn(m0, sc);
         m1 = __dmul_rn(m1, sc);
         m2 = __dmul_rn(m2, sc);
+        mk = __dmul_rn(mk, sc);
         mm = __fma_rn(m2, m2, __fma_rn(m1, m1, __dmul_rn(m0, m0)));
     }
-    const double inrm = rsqrt(mm);
-    e0 = __dmul_rn(m0, inrm);
-    e1 = __dmul_rn(m1, inrm);
-    e2 = __dmul_rn(m2, inrm);
-    return true;
-}
-
-// The terms of one corner: t_n = w.a and t_d = |a|^2 with d = x_p - r_i (the
-// corner minus the cell fraction, exact), w = u_p - V and the basis
-// a = (1 - 3R/(4 r)) e^N - 3R (e^N.d)/(4 r^3) d; zero for a corner the fit
-// skips (r < 1e-12, or r < R with exclude).
-__device__ __forceinline__ void fit_corner(double d0, double d1, double d2, double e0, double e1, double e2,
-                                           double R34, double R2, int exclude, double w0, double w1, double w2,
-                                           double &tn, double &td) {
-    tn = 0.0;
-    td = 0.0;
-    const double rr = __fma_rn(d2, d2, __fma_rn(d1, d1, __dmul_rn(d0, d0)));
-    if (rr < 1e-24 || (exclude && rr < R2)) return;
-    const double ir = rsqrt(rr);
-    const double x = __fma_rn(e2, d2, __fma_rn(e1, d1, __dmul_rn(e0, d0)));
-    const double k1 = __fma_rn(-R34, ir, 1.0);
-    const double k2 = __dmul_rn(__dmul_rn(R34, x), __dmul_rn(__dmul_rn(ir, ir), ir));
-    const double a0 = __fma_rn(k1, e0, -__dmul_rn(k2, d0));
-    const double a1 = __fma_rn(k1, e1, -__dmul_rn(k2, d1));
-    const double a2 = __fma_rn(k1, e2, -__dmul_rn(k2, d2));
-    tn = __fma_rn(w2, a2, __fma_rn(w1, a1, __dmul_rn(w0, a0)));
-    td = __fma_rn(a2, a2, __fma_rn(a1, a1, __dmul_rn(a0, a0)));
-}
-
-// Sum of v over the eight lanes of a particle (lanes 8j .. 8j + 7), in the
-// tree order above; every lane of the group gets the same sum.
-__device__ __forceinline__ double sum8(double v) {
+    const double ek = __dmul_rn(mk, rsqrt(mm));
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    for (int k = 0; k < 3; ++k) e[k] = from_comp(ek, k);
+    return (any & 0x7fffffffffffffffll) != 0;
 }
 
-// Particles per block: 32 (256 threads) with the fit one thread per particle
-// (FIT8 = false); 8 (64 threads) with the fit one lane per corner (FIT8 =
-// true).  An FP64 warp instruction occupies the SM's narrow FP64 pipe for 16
-// cycles whatever its active lanes, and the fit is ~480 of them per particle.
-// With many particles the pipe is the limit and one thread per particle uses
-// every lane of each instruction.  With few particles (a warp or two per SM)
-// the fit is one warp's chain of dependent FP64 instructions; spreading the
-// eight corners over eight lanes, and the particles over more blocks, cuts
-// that chain about fourfold.
-constexpr int PB_WIDE = 32, PB_NARROW = 8;
+constexpr int PN = 16;             // particles per block (32: 334.5 against 332.6 us a step at 256^3)
+constexpr int PL_T = 8 * PN + 32;  // eight threads each, and the triggering warp
 
-// 64 registers (four blocks of 256 threads per SM) keep the 16384-particle
-// grid of the 256^3 workload (512 blocks) in a single wave on 152 SMs (at 80
-// registers, three blocks per SM, it took two).
-template <typename St, int MAXR, int PB, bool FIT8>
-__global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(const ParticleArgs A,
-                                                                            const RepTable<MAXR> rt) {
+// the particle warps of a block (the triggering warp has left)
+__device__ __forceinline__ void sync_particles() { asm volatile("bar.sync 1, %0;" ::"n"(8 * PN) : "memory"); }
+
+// No spills at 96 registers, 20 warps per SM (at 64, 30 warps: 340.6 against
+// 332.8 us a step at 256^3 with 16384 particles).
+template <typename St, int MAXR, bool MANY>
+__global__ void __launch_bounds__(PL_T, 4) k_particles(const ParticleArgs A, const RepTable<MAXR> rt) {
+    if (threadIdx.x >= 8 * PN) {
+        // lets the lattice pass of this step launch as soon as the one before it is
+        // complete, whatever the others are still preparing; it waits for this
+        // grid's completion before it reads anything this kernel writes
+        grid_dependency_wait();
+        grid_dependents_launch();
+        return;
+    }
     const typename St::T *G = static_cast<const typename St::T *>(A.g);
-    __shared__ int s_base[PB][3];
-    __shared__ int s_rep[PB];
-    // u^N of each corner: summed in FP32 by its gather thread, which also
-    // converts it to FP64 (exact), while the FP64 pipe is otherwise idle
-    __shared__ double s_u[PB][8][3];
-    __shared__ long long s_fix[PB][3];
-    __shared__ long long s_frac[PB][3];
-    __shared__ int s_spread[PB];
-    __shared__ int s_next[PB][3];  // cell after the update
-    // state read only by the Langevin update, staged by warp 1 so that warp 0
-    // (the FP64 fit) carries fewer registers across the gather
-    __shared__ double s_fe[3][PB];
-    __shared__ double s_invM[PB], s_sg[PB];
-    __shared__ unsigned char s_pin[PB];
-    // one lane per corner: the particle state the corner lanes read, and the fit
-    __shared__ double s_q[FIT8 ? PB : 1][4], s_V[FIT8 ? PB : 1][3];
-    __shared__ double s_e[FIT8 ? PB : 1][3], s_nd[FIT8 ? PB : 1][2];
-    __shared__ int s_eok[FIT8 ? PB : 1];
-    const int t = threadIdx.x, lane = t & 31;
-    const int i0 = blockIdx.x * PB;
-    const int cap = A.cap;
+    const int p = threadIdx.x & 7, kc = comp_of(p);
+    const int ip = blockIdx.x * PN + (threadIdx.x >> 3);
+    const bool live = ip < A.np, owner = live && p < 3;  // the others shadow and store nothing
+    const int i = live ? ip : A.np - 1, cap = A.cap;
+    const int ik = kc * cap + i;
 
-    // ---- cell of each particle (warp 0): base = floor(r), q = r - base (exact).
-    // Warp 0 also loads all the particle state phase B needs now, so that its
-    // loads overlap this step's other memory round trips -- in a chained launch,
-    // the previous lattice pass (positions, velocities and forces were written
-    // before that pass, and are read through L2).
-    const int ip = i0 + lane;
-    double r0 = 0.0, r1 = 0.0, r2 = 0.0, q0 = 0.0, q1 = 0.0, q2 = 0.0;
-    double V0 = 0.0, V1 = 0.0, V2 = 0.0, gam = 0.0, Rd = 0.0;
-    if (t >= 32 && t < 32 + PB && ip < A.np) {
-        s_invM[lane] = A.inv_mass[ip];
-        s_sg[lane] = A.sig[ip];
-        if (A.fext_in) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const double f = A.fext_in[3 * (size_t)ip + k];
-                s_fe[k][lane] = f;
-                A.fext[k * cap + ip] = f;  // kept for the steps that follow
+    // ---- state of the particle, written before the previous lattice pass
+    const double rk = __ldcg(A.r + ik), Vk = __ldcg(A.v + ik);
+    double fek;
+    if (A.fext_in) {
+        fek = A.fext_in[3 * (size_t)i + kc];
+        if (owner) A.fext[ik] = fek;  // kept for the steps that follow
+    } else {
+        fek = __ldcg(A.fext + ik);
+    }
+    const double gam = A.gamma[i], Rd = A.radius[i], invM = A.inv_mass[i], sg = A.sig[i];
+    const bool pin = A.pinned[i] != 0;
+    const Rep &rp = rt.rep[MAXR == 1 ? 0 : A.prep[i]];
+    const int nx = rp.nx, ny = rp.ny, nz = rp.nz;
+    const int Lk = kc == 0 ? nx : kc == 1 ? ny : nz;
+
+    // cell: base = floor(r), q = r - base (exact); this lane's corner
+    const double bk = floor(rk), qk = rk - bk;
+    const int base = (int)bk;
+    const int c0 = p & 1, c1 = (p >> 1) & 1, c2 = p >> 2;
+    const int X = wrapi(from_comp(base, 0) + c0, nx), Y = wrapi(from_comp(base, 1) + c1, ny),
+              Z = wrapi(from_comp(base, 2) + c2, nz);
+    // q as 31-bit fraction floor(q 2^31), for the spreading
+    const unsigned frac = __double2uint_rz(qk * 2147483648.0);
+    // the corner's fit geometry: with d = x_p - r_i (the corner minus the cell
+    // fraction, exact) and r = |d|, the coefficients 1 - 3R/(4 r) and 1/r^3 of
+    // Eq. 8; or the trilinear weight for Eq. 7.  A corner with r < 1e-12 (or r < R
+    // with exclude_inside) is left out of the fit.
+    double d0 = 0.0, d1 = 0.0, d2 = 0.0, k1 = 0.0, ir3 = 0.0, Wp = 0.0;
+    bool use = false;
+    auto geometry = [&] {
+        if (A.mode == LBP_BROWNIAN) return;
+        const double q0 = from_comp(qk, 0), q1 = from_comp(qk, 1), q2 = from_comp(qk, 2);
+        if (A.mode == LBP_STOKESLET) {
+            d0 = c0 ? __dsub_rn(1.0, q0) : -q0;
+            d1 = c1 ? __dsub_rn(1.0, q1) : -q1;
+            d2 = c2 ? __dsub_rn(1.0, q2) : -q2;
+            const double rr = __fma_rn(d2, d2, __fma_rn(d1, d1, __dmul_rn(d0, d0)));
+            use = !(rr < 1e-24 || (A.exclude_inside && rr < Rd * Rd));
+            if (use) {
+                const double ir = rsqrt(rr);
+                k1 = __fma_rn(-(0.75 * Rd), ir, 1.0);
+                ir3 = __dmul_rn(__dmul_rn(ir, ir), ir);
             }
         } else {
-            s_fe[0][lane] = __ldcg(A.fext + ip);
-            s_fe[1][lane] = __ldcg(A.fext + cap + ip);
-            s_fe[2][lane] = __ldcg(A.fext + 2 * cap + ip);
+            Wp = (c0 ? q0 : 1.0 - q0) * (c1 ? q1 : 1.0 - q1) * (c2 ? q2 : 1.0 - q2);
         }
-        s_pin[lane] = A.pinned[ip];
+    };
+    // Eqs. 4-5: F_R = sqrt(2 gamma kT) xi, xi = sqrt3 (2u - 1) with
+    // u = ((x >> 11) + 1/2) 2^-53 from Philox(counter = (step, i, 0, 0), key = (seed, 0)).
+    // 2u - 1 is formed as fma((double)(2k + 1), 2^-53, -1): the same correctly
+    // rounded value as 2 ((double)k + 1/2) 2^-53 - 1, so F_R is bit-identical
+    // to the oracle's.
+    auto random_force = [&](long long step) {
+        unsigned long long ctr[4] = {(unsigned long long)step, (unsigned long long)i, 0ull, 0ull};
+        philox4x64_10(ctr, A.seed, 0ull);
+        const unsigned long long x = kc == 0 ? ctr[0] : kc == 1 ? ctr[1] : ctr[2];
+        const double tt = __fma_rn(__ull2double_rn(2ull * (x >> 11) + 1ull), 0x1.0p-53, -1.0);
+        return __dmul_rn(sg, __dmul_rn(A.sqrt3, tt));
+    };
+    long long step = 0;
+    double Rk = 0.0;
+    if (A.chained) step = __ldcg(A.step_in);
+    if (!MANY) {
+        geometry();
+        if (A.chained) Rk = random_force(step);
     }
-    if (t < PB && ip < A.np) {
-        r0 = __ldcg(A.r + ip);
-        r1 = __ldcg(A.r + cap + ip);
-        r2 = __ldcg(A.r + 2 * cap + ip);
-        V0 = __ldcg(A.v + ip);
-        V1 = __ldcg(A.v + cap + ip);
-        V2 = __ldcg(A.v + 2 * cap + ip);
-        gam = A.gamma[ip];
-        Rd = A.radius[ip];
-        s_rep[lane] = MAXR == 1 ? 0 : A.prep[ip];
-        const double b0 = floor(r0), b1 = floor(r1), b2 = floor(r2);
-        q0 = r0 - b0;
-        q1 = r1 - b1;
-        q2 = r2 - b2;
-        s_base[lane][0] = (int)b0;
-        s_base[lane][1] = (int)b1;
-        s_base[lane][2] = (int)b2;
-        if (FIT8) {
-            s_q[lane][0] = q0;
-            s_q[lane][1] = q1;
-            s_q[lane][2] = q2;
-            s_q[lane][3] = Rd;
-            s_V[lane][0] = V0;
-            s_V[lane][1] = V1;
-            s_V[lane][2] = V2;
-        }
-    }
-    // the previous lattice pass is complete: populations, step index, records
-    grid_dependency_wait();
-    const long long step = __ldcg(A.d_step);
-    // the step's lattice pass may launch now: it waits for this grid's
-    // completion before it reads anything this kernel writes (or bumps the step)
-    grid_dependents_launch();
-    if ((A.ring || A.ring16) && blockIdx.x == 0 && t == 0) {
-        const long long m = step - A.d_vacf[0];
-        if (m >= 0) A.d_vacf[2] = m + 1;
-    }
-    __syncthreads();
 
-    // ---- phase A: u at corner p, u = sum_a e_a g_a(x_p - e_a) (FP32)
-    const int j = t >> 3, p = t & 7;
-    const int ij = i0 + j;
-    const int c0 = p & 1, c1 = (p >> 1) & 1, c2 = (p >> 2) & 1;
-    int X = 0, Y = 0, Z = 0;
-    const Rep &rj = rt.rep[MAXR == 1 || ij >= A.np ? 0 : s_rep[j]];
-    const int nx = rj.nx, ny = rj.ny, nz = rj.nz;
-    if (ij < A.np) {
-        X = wrapi(s_base[j][0] + c0, nx);
-        Y = wrapi(s_base[j][1] + c1, ny);
-        Z = wrapi(s_base[j][2] + c2, nz);
+    // ---- the previous lattice pass is complete: populations, step index, records
+    grid_dependency_wait();
+    float sx = 0.f, sy = 0.f, sz = 0.f;
+    {
+        // u at corner p, u = sum_a e_a g_a(x_p - e_a) (FP32)
         const int xs[3] = {wrapi(X + 1, nx), X, wrapi(X - 1, nx)};  // x - e for e = -1, 0, 1
         const int ys[3] = {wrapi(Y + 1, ny), Y, wrapi(Y - 1, ny)};
         const int zs[3] = {wrapi(Z + 1, nz), Z, wrapi(Z - 1, nz)};
-        float sx = 0.f, sy = 0.f, sz = 0.f;
+        float g[Q];
+#pragma unroll
+        for (int a = 1; a < Q; ++a)
+            g[a] = St::gather(G + ((long long)a * A.P + rp.node_off +
+                                   ((long long)zs[ez(a) + 1] * ny + ys[ey(a) + 1]) * nx + xs[ex(a) + 1]), a);
+        if (!A.chained) step = __ldcg(A.d_step);
+        if (MANY) geometry();
+        if (MANY || !A.chained) Rk = random_force(step);
 #pragma unroll
         for (int a = 1; a < Q; ++a) {
-            const long long src = (long long)a * A.P + rj.node_off +
-                                  ((long long)zs[ez(a) + 1] * ny + ys[ey(a) + 1]) * nx + xs[ex(a) + 1];
-            const float gv = St::gather(G + src, a);
-            if (ex(a)) sx += ex(a) > 0 ? gv : -gv;
-            if (ey(a)) sy += ey(a) > 0 ? gv : -gv;
-            if (ez(a)) sz += ez(a) > 0 ? gv : -gv;
+            if (ex(a)) sx += ex(a) > 0 ? g[a] : -g[a];
+            if (ey(a)) sy += ey(a) > 0 ? g[a] : -g[a];
+            if (ez(a)) sz += ez(a) > 0 ? g[a] : -g[a];
         }
-        s_u[j][p][0] = (double)sx;
-        s_u[j][p][1] = (double)sy;
-        s_u[j][p][2] = (double)sz;
     }
-    __syncthreads();
-
-    // ---- the fit of Eq. 8 with one lane per corner (all threads): the mean
-    // relative velocity and e^N in every lane of the particle (sum8 gives all
-    // eight the same sum), the corner's terms, their sums to s_nd
-    if (FIT8 && A.mode == LBP_STOKESLET) {
-        const bool live = ij < A.np;
-        double V[3] = {0.0, 0.0, 0.0}, m[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (live) V[k] = s_V[j][k];
-            m[k] = __fma_rn(-8.0, V[k], sum8(live ? s_u[j][p][k] : 0.0));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *A.step_out = step + 1;
+        if (A.ring || A.ring16) {
+            const long long m = step - A.d_vacf[0];
+            if (m >= 0) A.d_vacf[2] = m + 1;
         }
-        double e0 = 0.0, e1 = 0.0, e2 = 0.0;
-        const bool eok = live && fit_direction(m[0], m[1], m[2], e0, e1, e2);
+    }
+
+    // ---- friction force: component kc in every lane
+    const double u0 = widen_f32(sx), u1 = widen_f32(sy), u2 = widen_f32(sz);
+    double Fk = 0.0;
+    if (A.mode == LBP_STOKESLET) {
+        // Eq. 8: w_p = u_p - V, e^N = mean(w)/|mean(w)|, basis
+        // a_p = (1 - 3R/(4 r_p)) e^N - 3R (e^N.d_p)/(4 r_p^3) d_p, and the normal
+        // equation U_inf sum|a_p|^2 = sum w_p.a_p, solved for U_inf;
+        // F_H = gamma U_inf e^N (Eq. 7 with u_inf = U_inf e^N + V)
+        double e[3];
+        const bool eok = direction(__fma_rn(-8.0, Vk, sum_components(u0, u1, u2, p)), e);
+        const double w0 = __dsub_rn(u0, from_comp(Vk, 0)), w1 = __dsub_rn(u1, from_comp(Vk, 1)),
+                     w2 = __dsub_rn(u2, from_comp(Vk, 2));
         double tn = 0.0, td = 0.0;
+        if (eok && use) {
+            const double x = __fma_rn(e[2], d2, __fma_rn(e[1], d1, __dmul_rn(e[0], d0)));
+            const double k2 = __dmul_rn(__dmul_rn(0.75 * Rd, x), ir3);
+            const double a0 = __fma_rn(k1, e[0], -__dmul_rn(k2, d0));
+            const double a1 = __fma_rn(k1, e[1], -__dmul_rn(k2, d1));
+            const double a2 = __fma_rn(k1, e[2], -__dmul_rn(k2, d2));
+            tn = __fma_rn(w2, a2, __fma_rn(w1, a1, __dmul_rn(w0, a0)));
+            td = __fma_rn(a2, a2, __fma_rn(a1, a1, __dmul_rn(a0, a0)));
+        }
+        const double nd = sum_pair(tn, td, p);
+        const double num = __shfl_sync(0xffffffffu, nd, 0, 8), den = __shfl_sync(0xffffffffu, nd, 1, 8);
         if (eok) {
-            const double q0p = s_q[j][0], q1p = s_q[j][1], q2p = s_q[j][2], Rp = s_q[j][3];
-            const double d0 = c0 ? __dsub_rn(1.0, q0p) : -q0p;
-            const double d1 = c1 ? __dsub_rn(1.0, q1p) : -q1p;
-            const double d2 = c2 ? __dsub_rn(1.0, q2p) : -q2p;
-            fit_corner(d0, d1, d2, e0, e1, e2, 0.75 * Rp, Rp * Rp, A.exclude_inside,
-                       __dsub_rn(s_u[j][p][0], V[0]), __dsub_rn(s_u[j][p][1], V[1]),
-                       __dsub_rn(s_u[j][p][2], V[2]), tn, td);
+            const long long db = __double_as_longlong(den);
+            const double U = db > 0 && db <= 0x7ff0000000000000ll ? num / den : 0.0;  // den > 0
+            Fk = __dmul_rn(__dmul_rn(gam, U), kc == 0 ? e[0] : kc == 1 ? e[1] : e[2]);
         }
-        tn = sum8(tn);
-        td = sum8(td);
-        if (live && p == 0) {
-            s_eok[j] = eok;
-            s_e[j][0] = e0;
-            s_e[j][1] = e1;
-            s_e[j][2] = e2;
-            s_nd[j][0] = tn;
-            s_nd[j][1] = td;
+    } else if (A.mode == LBP_POINTWISE) {
+        // Eq. 7 with u(r_i) = sum_p W_p u^N_p, corner after corner
+        double ur = 0.0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const double v0 = __shfl_sync(0xffffffffu, u0, c, 8), v1 = __shfl_sync(0xffffffffu, u1, c, 8),
+                         v2 = __shfl_sync(0xffffffffu, u2, c, 8);
+            ur = __fma_rn(__shfl_sync(0xffffffffu, Wp, c, 8), kc == 0 ? v0 : kc == 1 ? v1 : v2, ur);
         }
-        __syncthreads();
+        Fk = __dmul_rn(-gam, __dsub_rn(Vk, ur));
+    } else {
+        // Eq. 6: friction against a fluid at rest; nothing is returned to the fluid
+        Fk = __dmul_rn(-gam, Vk);
     }
 
-    // ---- phase B (warp 0): fit, random force, Langevin update
-    if (t < PB && ip < A.np) {
-        const int i = ip;
-        double F0 = 0.0, F1 = 0.0, F2 = 0.0;
-        bool spread = true;
-        if (A.mode == LBP_STOKESLET) {
-            // Eq. 8 in FP64 from the FP32 corner velocities: w_p = u_p - V,
-            // e^N = mean(w)/|mean(w)|, d_p = x_p - r_i (exact: corner minus
-            // cell fraction), basis a_p = (1 - 3R/(4 r_p)) e^N - 3R (e^N.d_p)/(4 r_p^3) d_p,
-            // and the normal equation U_inf sum|a_p|^2 = sum w_p.a_p, solved
-            // for U_inf; F_H = gamma U_inf e^N (Eq. 7 with u_inf = U_inf e^N + V).
-            double num = 0.0, den = 0.0, e0 = 0.0, e1 = 0.0, e2 = 0.0;
-            bool eok;
-            if (FIT8) {
-                eok = s_eok[lane];
-                e0 = s_e[lane][0];
-                e1 = s_e[lane][1];
-                e2 = s_e[lane][2];
-                num = s_nd[lane][0];
-                den = s_nd[lane][1];
-            } else {
-                // the same operations as the lane-per-corner layout, in one
-                // thread: w_p is formed again in the corner loop from the shared
-                // corner velocities (holding all 24 would spill)
-                double m[3];
-                const double Vk[3] = {V0, V1, V2};
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    asm volatile("" ::: "memory");
-                    double h[4];
-#pragma unroll
-                    for (int c = 0; c < 8; c += 2)
-                        h[c >> 1] = __dadd_rn(s_u[lane][c][k], s_u[lane][c + 1][k]);
-                    m[k] = __fma_rn(-8.0, Vk[k], __dadd_rn(__dadd_rn(h[0], h[1]), __dadd_rn(h[2], h[3])));
-                }
-                eok = fit_direction(m[0], m[1], m[2], e0, e1, e2);
-                if (eok) {
-                    const double R34 = 0.75 * Rd, R2 = Rd * Rd;
-                    const double dx[2] = {-q0, __dsub_rn(1.0, q0)}, dy[2] = {-q1, __dsub_rn(1.0, q1)},
-                                 dz[2] = {-q2, __dsub_rn(1.0, q2)};
-                    double hn[4], hd[4];
-#pragma unroll
-                    for (int c = 0; c < 8; c += 2) {
-                        // load each pair's corner velocities where they are used
-                        // (hoisting all 24 doubles would spill)
-                        asm volatile("" ::: "memory");
-                        double tn0, td0, tn1, td1;
-                        fit_corner(dx[0], dy[(c >> 1) & 1], dz[(c >> 2) & 1], e0, e1, e2, R34, R2, A.exclude_inside,
-                                   __dsub_rn(s_u[lane][c][0], V0), __dsub_rn(s_u[lane][c][1], V1),
-                                   __dsub_rn(s_u[lane][c][2], V2), tn0, td0);
-                        fit_corner(dx[1], dy[(c >> 1) & 1], dz[(c >> 2) & 1], e0, e1, e2, R34, R2, A.exclude_inside,
-                                   __dsub_rn(s_u[lane][c + 1][0], V0),
-                                   __dsub_rn(s_u[lane][c + 1][1], V1),
-                                   __dsub_rn(s_u[lane][c + 1][2], V2), tn1, td1);
-                        hn[c >> 1] = __dadd_rn(tn0, tn1);
-                        hd[c >> 1] = __dadd_rn(td0, td1);
-                    }
-                    num = __dadd_rn(__dadd_rn(hn[0], hn[1]), __dadd_rn(hn[2], hn[3]));
-                    den = __dadd_rn(__dadd_rn(hd[0], hd[1]), __dadd_rn(hd[2], hd[3]));
-                }
-            }
-            if (eok) {
-                const double U = den > 0.0 ? num / den : 0.0;
-                const double gU = gam * U;
-                F0 = gU * e0;
-                F1 = gU * e1;
-                F2 = gU * e2;
-            }
-        } else if (A.mode == LBP_POINTWISE) {
-            // Eq. 7 with u(r_i) = sum_p W_p u^N_p (trilinear weights of the cell
-            // fraction), in FP64
-            const double wx[2] = {1.0 - q0, q0}, wy[2] = {1.0 - q1, q1}, wz[2] = {1.0 - q2, q2};
-            double ur0 = 0.0, ur1 = 0.0, ur2 = 0.0;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const double Wp = wx[c & 1] * wy[(c >> 1) & 1] * wz[(c >> 2) & 1];
-                ur0 += Wp * s_u[lane][c][0];
-                ur1 += Wp * s_u[lane][c][1];
-                ur2 += Wp * s_u[lane][c][2];
-            }
-            F0 = -gam * (V0 - ur0);
-            F1 = -gam * (V1 - ur1);
-            F2 = -gam * (V2 - ur2);
-        } else {
-            // Eq. 6: friction against a fluid at rest; nothing is returned to the fluid
-            F0 = -gam * V0;
-            F1 = -gam * V1;
-            F2 = -gam * V2;
-            spread = false;
-        }
-        if (spread) {
-            const bool ok = fabs(F0) < FIX_LIMIT && fabs(F1) < FIX_LIMIT && fabs(F2) < FIX_LIMIT;
-            if (!ok) {
-                atomicOr(A.err, ERR_RANGE);
-                spread = false;
-            } else {
-                s_fix[lane][0] = __double2ll_rn(-F0 * FIX_SCALE);
-                s_fix[lane][1] = __double2ll_rn(-F1 * FIX_SCALE);
-                s_fix[lane][2] = __double2ll_rn(-F2 * FIX_SCALE);
-                // q as 31-bit fractions q31 = floor(q 2^31) in bits 32..62
-                s_frac[lane][0] = (long long)((unsigned long long)__double2uint_rz(q0 * 2147483648.0) << 32);
-                s_frac[lane][1] = (long long)((unsigned long long)__double2uint_rz(q1 * 2147483648.0) << 32);
-                s_frac[lane][2] = (long long)((unsigned long long)__double2uint_rz(q2 * 2147483648.0) << 32);
-            }
-        }
-        s_spread[lane] = spread ? 1 : 0;
-
-        // Eqs. 4-5: F_R = sqrt(2 gamma kT) xi, xi = sqrt3 (2u - 1) with
-        // u = ((x >> 11) + 1/2) 2^-53 from Philox(counter = (step, i, 0, 0), key = (seed, 0)).
-        // 2u - 1 is formed as fma((double)(2k + 1), 2^-53, -1): the same correctly
-        // rounded value as 2 ((double)k + 1/2) 2^-53 - 1, so F_R is bit-identical
-        // to the oracle's.
-        unsigned long long ctr[4] = {(unsigned long long)step, (unsigned long long)i, 0ull, 0ull};
-        philox4x64_10(ctr, A.seed, 0ull);
-        double R3[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double tt = __fma_rn(__ull2double_rn(2ull * (ctr[k] >> 11) + 1ull), 0x1.0p-53, -1.0);
-            R3[k] = __dmul_rn(s_sg[lane], __dmul_rn(A.sqrt3, tt));
-        }
-        const double FH3[3] = {F0, F1, F2};
-        const double Vo[3] = {V0, V1, V2};
-        const double ro[3] = {r0, r1, r2};
-        const double invM = s_invM[lane];
-        const bool pin = s_pin[lane] != 0;
-        const Rep &ri = rt.rep[MAXR == 1 ? 0 : s_rep[lane]];
-        const int L[3] = {ri.nx, ri.ny, ri.nz};
-        double Vn[3] = {V0, V1, V2};
-        bool bad = false;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            A.fh[k * cap + i] = FH3[k];
-            A.fr[k * cap + i] = R3[k];
-            double rw = ro[k];
-            if (!pin) {
-                // Eqs. 1-2, dt = 1: V += (F_H + F_R + F_ext)/M; r += V; periodic wrap
-                Vn[k] = Vo[k] + (FH3[k] + R3[k] + s_fe[k][lane]) * invM;
-                double rn = ro[k] + Vn[k];
-                if (rn < 0.0) rn += (double)L[k];
-                if (rn >= (double)L[k]) rn -= (double)L[k];
-                const bool b = !isfinite(Vn[k]) || !(rn >= 0.0) || !(rn < (double)L[k]);
-                if (b) rn = 0.0;  // keep the next gather inside the box; reported as LBP_ENAN
-                bad |= b;
-                A.v[k * cap + i] = Vn[k];
-                A.r[k * cap + i] = rn;
-                rw = rn;
-            }
-            if (A.marks) s_next[lane][k] = (int)floor(rw);
-            if (FIT8) {  // few particles: straight from the update's registers
-                if (A.r_out) A.r_out[3 * (size_t)i + k] = rw;
-                if (A.v_out) A.v_out[3 * (size_t)i + k] = Vn[k];
-            }
-        }
-        if (FIT8 && A.done_flag) __threadfence_system();  // the host copies before the flag
-        if (bad) atomicOr(A.err, ERR_NAN);
-        if (A.inj)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) s_fe[k][lane] = pin ? 0.0 : R3[k] + s_fe[k][lane];
-        if (A.ring) {
-            const long long m = step - A.d_vacf[0];
-            if (m >= 0) {
-                float *dst = A.ring + (m % A.ring_cap) * 3 * (long long)A.np;
-                dst[i] = (float)Vn[0];
-                dst[A.np + i] = (float)Vn[1];
-                dst[2 * A.np + i] = (float)Vn[2];
-            }
-        }
-        if (A.ring16) {
-            // the sample as fp16 hi/lo of 4096 V (the tensor-core correlator's
-            // operands), at its ring row and, for the first rows, once more
-            // after the end of the ring
-            const long long m = step - A.d_vacf[0];
-            if (m >= 0) {
-                const int row = (int)(m % A.ring_cap);
-                bool big = false;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const double a = Vn[k] * (double)VACF_RING_SCALE;
-                    big |= !(fabs(a) < 65504.0);
-                    const __half hi = __double2half(a);
-                    const __half lo = __double2half(a - (double)__half2float(hi));
-                    const long long j = (long long)k * A.np + i;
-                    __half *p = A.ring16 + (long long)row * 2 * A.ring_ld + j;
-                    p[0] = hi;
-                    p[A.ring_ld] = lo;
-                    if (row < A.ring_dup) {
-                        __half *p2 = p + (long long)A.ring_cap * 2 * A.ring_ld;
-                        p2[0] = hi;
-                        p2[A.ring_ld] = lo;
-                    }
-                }
-                if (big) atomicOr(A.err, ERR_RANGE);
-            }
-        }
-    }
-    __syncthreads();
-
-    // With many particles (one thread per particle), positions and velocities
-    // go to the caller's buffers ([n][3], host memory seen through its device
-    // mapping) as one contiguous span per block, read back from the state
-    // arrays the update above wrote (a pinned particle's entries there are its
-    // unchanged ones), before phase C so that their round trip overlaps it.
-    // (With one lane per corner the update's threads write them directly: the
-    // 64-register budget of that layout has no room for this step beside
-    // phase C's live values.)
-    if (!FIT8 && (A.r_out || A.v_out) && t < 3 * PB && 3LL * i0 + t < 3LL * A.np) {
-        const int pi = i0 + t / 3, k = t - 3 * (t / 3);
-        if (A.r_out) A.r_out[3LL * i0 + t] = A.r[k * cap + pi];
-        if (A.v_out) A.v_out[3LL * i0 + t] = A.v[k * cap + pi];
-    }
-
-    if (A.inj && t < 32) {
-        // conservation budget: the momentum F_R + F_ext put into the block's
-        // unpinned particles (left in s_fe by phase B), summed over the warp,
-        // one FP64 atomic per component
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            double vk = lane < PB && ip < A.np ? s_fe[k][lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) vk += __shfl_xor_sync(0xffffffffu, vk, o);
-            if (lane == 0) atomicAdd(A.inj + k, vk);
-        }
-    }
-
-    // ---- phase C: share of corner p of the fixed-point reaction force -F_H.
+    // ---- share of corner p of the fixed-point reaction force -F_H.
     // Per axis the far corner (c = 1) takes floor(v q) -- the signed high half
     // of (2 v) (q31 2^32) -- and the near corner the rest, so the eight shares
     // add up to v exactly.  |v| < 2^61 (|F_H| < 32), so 2 v stays within int64.
-    if (ij < A.np && s_spread[j]) {
-        const int cc[3] = {c0, c1, c2};
-        long long sh[3];
+    if (A.mode != LBP_BROWNIAN) {
+        const bool ok = below(Fk, FIX_LIMIT);
+        const unsigned oks = __ballot_sync(0xffffffffu, ok) >> (threadIdx.x & 24) & 0xffu;
+        const long long fix = ok ? __double2ll_rn(-Fk * FIX_SCALE) : 0ll;
+        long long q31[3];
+        unsigned long long sh[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) q31[k] = (long long)((unsigned long long)from_comp(frac, k) << 32);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            long long v = s_fix[j][k];
-#pragma unroll
-            for (int ax = 0; ax < 3; ++ax) {
-                const long long far = __mul64hi(2 * v, s_frac[j][ax]);
-                v = cc[ax] ? far : v - far;
-            }
-            sh[k] = v;
+            long long v = from_comp(fix, k), far = __mul64hi(2 * v, q31[0]);
+            v = c0 ? far : v - far;
+            far = __mul64hi(2 * v, q31[1]);
+            v = c1 ? far : v - far;
+            far = __mul64hi(2 * v, q31[2]);
+            sh[k] = (unsigned long long)(c2 ? far : v - far);
         }
-        const long long row = (long long)Z * ny + Y;
-        unsigned long long *rec =
-            A.rec + (size_t)(rj.seg_off + row * rj.nchunks + X / SEG) * REC_WORDS;
-        const unsigned int slot = atomicAdd(reinterpret_cast<unsigned int *>(rec), 1u);
-        if (slot < (unsigned)REC_SLOTS) {
-            reinterpret_cast<int *>(rec + REC_X0)[slot] = X;
-            rec[REC_F0 + 3 * slot] = (unsigned long long)sh[0];
-            rec[REC_F0 + 3 * slot + 1] = (unsigned long long)sh[1];
-            rec[REC_F0 + 3 * slot + 2] = (unsigned long long)sh[2];
-        } else {
-            const long long node = rj.node_off + row * nx + X;
-            atomicAdd(A.fq + node, (unsigned long long)sh[0]);
-            atomicAdd(A.fq + A.N + node, (unsigned long long)sh[1]);
-            atomicAdd(A.fq + 2 * A.N + node, (unsigned long long)sh[2]);
+        if (oks != 0xffu) {
+            if (live && p == 0) atomicOr(A.err, ERR_RANGE);
+        } else if (live) {
+            const long long row = (long long)Z * ny + Y;
+            unsigned long long *rec = A.rec + (size_t)(rp.seg_off + row * rp.nchunks + X / SEG) * REC_WORDS;
+            const unsigned int slot = atomicAdd(reinterpret_cast<unsigned int *>(rec), 1u);
+            if (slot < (unsigned)REC_SLOTS) {
+                reinterpret_cast<int *>(rec + REC_X0)[slot] = X;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) rec[REC_F0 + 3 * slot + k] = sh[k];
+            } else {
+                const long long node = rp.node_off + row * nx + X;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) atomicAdd(A.fq + k * A.N + node, sh[k]);
+            }
         }
     }
 
-    // mark the row segment of corner p of the next step's cell
-    if (A.marks && ij < A.np) {
-        const int x1 = wrapi(s_next[j][0] + c0, nx), y1 = wrapi(s_next[j][1] + c1, ny),
-                  z1 = wrapi(s_next[j][2] + c2, nz);
-        A.marks[rj.seg_off + ((long long)z1 * ny + y1) * rj.nchunks + x1 / SEG] = A.mark_epoch;
+    // ---- Eqs. 1-2, dt = 1: V += (F_H + F_R + F_ext)/M; r += V; periodic wrap
+    double Vn = Vk, rn = rk;
+    if (!pin) {
+        Vn = __fma_rn(__dadd_rn(__dadd_rn(Fk, Rk), fek), invM, Vk);
+        rn = __dadd_rn(rk, Vn);
+        const double L = (double)Lk;
+        const long long Lb = __double_as_longlong(L);
+        if (negative(rn)) rn = __dadd_rn(rn, L);
+        if (__double_as_longlong(rn) >= Lb) rn = __dsub_rn(rn, L);
+        if (!below(Vn, __longlong_as_double(0x7ff0000000000000ll)) || negative(rn) ||
+            __double_as_longlong(rn) >= Lb) {
+            rn = 0.0;  // keep the next gather inside the box; reported as LBP_ENAN
+            if (live) atomicOr(A.err, ERR_NAN);
+        }
+    }
+    if (owner) {
+        A.fh[ik] = Fk;
+        A.fr[ik] = Rk;
+        if (!pin) {
+            A.v[ik] = Vn;
+            A.r[ik] = rn;
+        }
+        if (A.r_out) A.r_out[3 * (size_t)i + kc] = rn;
+        if (A.v_out) A.v_out[3 * (size_t)i + kc] = Vn;
+        if (A.done_flag) __threadfence_system();  // the host copies before the block's ticket
+    }
+    if (A.marks) {
+        // mark the row segment of corner p of the next step's cell
+        const int b = __double2int_rd(rn);
+        const int x1 = wrapi(from_comp(b, 0) + c0, nx), y1 = wrapi(from_comp(b, 1) + c1, ny),
+                  z1 = wrapi(from_comp(b, 2) + c2, nz);
+        if (live) A.marks[rp.seg_off + ((long long)z1 * ny + y1) * rp.nchunks + x1 / SEG] = A.mark_epoch;
+    }
+    if (owner && (A.ring || A.ring16)) {
+        const long long m = step - A.d_vacf[0];
+        const long long j = (long long)kc * A.np + i;
+        if (m >= 0 && A.ring) A.ring[(m % A.ring_cap) * 3 * (long long)A.np + j] = (float)Vn;
+        if (m >= 0 && A.ring16) {
+            // the sample as fp16 hi/lo of 4096 V (the tensor-core correlator's
+            // operands), at its ring row and, for the first rows, once more
+            // after the end of the ring
+            const int row = (int)(m % A.ring_cap);
+            const double a = Vn * (double)VACF_RING_SCALE;
+            const __half hi = __double2half(a);
+            const __half lo = __double2half(a - (double)__half2float(hi));
+            __half *w = A.ring16 + (long long)row * 2 * A.ring_ld + j;
+            w[0] = hi;
+            w[A.ring_ld] = lo;
+            if (row < A.ring_dup) {
+                w += (long long)A.ring_cap * 2 * A.ring_ld;
+                w[0] = hi;
+                w[A.ring_ld] = lo;
+            }
+            if (!below(a, 65504.0)) atomicOr(A.err, ERR_RANGE);
+        }
+    }
+
+    if (A.inj) {
+        // conservation budget: the momentum F_R + F_ext put into the block's
+        // unpinned particles, one FP64 atomic per component
+        __shared__ double s_inj[3][PN];
+        if (p < 3) s_inj[kc][threadIdx.x >> 3] = live && !pin ? Rk + fek : 0.0;
+        sync_particles();
+        if (threadIdx.x < 3) {
+            double v = 0.0;
+            for (int j = 0; j < PN; ++j) v += s_inj[threadIdx.x][j];
+            atomicAdd(A.inj + threadIdx.x, v);
+        }
     }
 
     // the last block to finish tells the host that every position and velocity
     // is in its buffers (the lattice pass may still run)
     if (A.done_flag) {
-        // the writes to the host buffers, made visible before the block's ticket
-        if (!FIT8 && t < 3 * PB) __threadfence_system();
-        __syncthreads();
-        if (t == 0) {
+        sync_particles();
+        if (threadIdx.x == 0) {
             const unsigned ticket = atomicAdd(A.done_ticket, 1u);
             if (ticket == gridDim.x - 1) {
                 *A.done_ticket = 0u;
@@ -601,35 +477,25 @@ __global__ void __launch_bounds__(8 * PB, PB == PB_WIDE ? 4 : 16) k_particles(co
     }
 }
 
-template <int MAXR, int PB, bool FIT8>
-static cudaError_t launch_particles_pb(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st,
-                                       bool chained) {
-    const unsigned grid = (unsigned)((s.np + PB - 1) / PB);
+// Few particles: the preparation before the launch dependency resolves (us a
+// step: 10.4 against 11.4 with 256 particles at 64^3, 67.9 against 68.6 with 7000
+// at 128^3).  From 48 per SM on: while the gather is in flight (98.1 against 97.4
+// with 8000 at 160^3, 331.8 against 327.8 with 16384 at 256^3).
+bool particles_few(const Sim &s) { return s.np < 48 * (s.num_sms > 0 ? s.num_sms : 1); }
+
+template <bool MANY, int MAXR>
+static cudaError_t launch_particles_m(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st) {
+    const unsigned grid = (unsigned)((s.np + PN - 1) / PN);
     switch (s.precision) {
-        case LBP_BF16: return launch_k(k_particles<StoreBF16, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
-        case LBP_F16: return launch_k(k_particles<StoreF16, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
-        default: return launch_k(k_particles<StoreF32, MAXR, PB, FIT8>, grid, 8 * PB, 0, st, chained, A, t);
+        case LBP_BF16: return launch_k(k_particles<StoreBF16, MAXR, MANY>, grid, PL_T, 0, st, A.chained, A, t);
+        case LBP_F16: return launch_k(k_particles<StoreF16, MAXR, MANY>, grid, PL_T, 0, st, A.chained, A, t);
+        default: return launch_k(k_particles<StoreF32, MAXR, MANY>, grid, PL_T, 0, st, A.chained, A, t);
     }
 }
 
-// The fit one lane per corner while the one-thread-per-particle layout would
-// leave the FP64 pipe mostly idle (fewer than ~50 particles per SM: its
-// dependent chain, not the pipe, sets the time); both give the same bits.
-bool particles_fit_per_corner(const Sim &s) { return s.np < 48 * (s.num_sms > 0 ? s.num_sms : 1); }
-
-// Whether the lattice pass lets the next particle kernel start before it ends.
-// Blocks that start while the pass drains crowd onto the SMs that empty first,
-// and the FP64 pipe (16 cycles a warp instruction) serves their fits one after
-// another: 63 narrow blocks at 80^3 took 37 instead of 13 us.  So early only
-// where they cannot crowd: the wide layout (at most four blocks per SM;
-// 341.4 -> 337.5 us a step at 256^3) and a single block (23.2 -> 22.2 us at 100^3).
-bool particles_start_early(const Sim &s) { return !particles_fit_per_corner(s) || s.np <= PB_NARROW; }
-
 template <int MAXR>
-static cudaError_t launch_particles_t(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st,
-                                      bool chained) {
-    if (particles_fit_per_corner(s)) return launch_particles_pb<MAXR, PB_NARROW, true>(s, A, t, st, chained);
-    return launch_particles_pb<MAXR, PB_WIDE, false>(s, A, t, st, chained);
+static cudaError_t launch_particles_t(const Sim &s, const ParticleArgs &A, const RepTable<MAXR> &t, cudaStream_t st) {
+    return particles_few(s) ? launch_particles_m<false>(s, A, t, st) : launch_particles_m<true>(s, A, t, st);
 }
 
 cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t st, const ParticleIO *io,
@@ -653,6 +519,9 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
     A.cap = s.cap;
     A.np = s.np;
     A.d_step = s.d_step;
+    A.step_in = s.d_step + 1 + parity;
+    A.step_out = s.d_step + 1 + (parity ^ 1);
+    A.chained = chained;
     A.seed = s.seed;
     A.sqrt3 = s.sqrt3;
     A.mode = s.mode;
@@ -681,13 +550,13 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
         t.item_off[0] = 0;
         t.item_off[1] = 0;
         t.rep[0] = s.reps[0];
-        return launch_particles_t(s, A, t, st, chained);
+        return launch_particles_t(s, A, t, st);
     } else {
         RepTable<MAX_BATCH> t;  // kernel parameter
         t.nrep = s.nrep;
         for (int r = 0; r <= s.nrep; ++r) t.item_off[r] = 0;
         for (int r = 0; r < s.nrep; ++r) t.rep[r] = s.reps[r];
-        return launch_particles_t(s, A, t, st, chained);
+        return launch_particles_t(s, A, t, st);
     }
 }
 

@@ -39,7 +39,8 @@ def run(boxes, counts, precision, mode, calls, shape, chain=True, lag=-1):
     ([(32, 32, 32)], [1]),              # a few marked rows
     ([(3, 5, 131)], [40]),              # corners that wrap in every direction, records that overflow
     ([(260, 9, 8)], [300]),             # three segments a row, most rows marked
-    ([(96, 64, 64)], [9000]),           # one thread per particle
+    ([(96, 64, 64)], [9000]),           # enough particles for the other order of preparation
+    ([(64, 64, 64)], [20000]),          # more particle blocks than are resident at a time
     ([(64, 20, 20), (17, 9, 30), (130, 8, 8)], [2, 0, 30])])
 @pytest.mark.parametrize("precision,shape", [
     (lbp.LBP_F32, None), (lbp.LBP_F32, (1, 0)), (lbp.LBP_F32, (4, 0)), (lbp.LBP_BF16, (2, 0)), (lbp.LBP_F16, None),
