@@ -14,17 +14,26 @@
 // these kernels produce dL/dfhat^{n-1}, dL/dV^n, dL/dr^n and add this step's
 // share of dL/domega, dL/dgamma_i, dL/dR_i, dL/dM_i and dL/dkT.
 //
-// k_adj_gather + k_adj_fp64 : eight threads per particle gather u(x_p) and
-//   lam_F(x_p) = sum_a 3 w_a e_a lam_a(x_p) at its corners (the adjoint of the
-//   body-force term) into a small scratch array; then one thread per particle,
-//   in 64-thread blocks so that many warps share each SM's FP64 pipe (the FP64
-//   chain is long and latency-bound), re-evaluates the particle's forward step
-//   in FP64 from the recorded state and runs
-//   the chain rule backwards through the update, the random force, the
-//   spreading weights and the Stokeslet fit.  What the fit sends back to the
-//   fluid is lam_u(x_p), the adjoint of the node velocity at each corner: it
-//   is appended, as (x, 3 FP64 values), to the 256-byte record of the corner's
-//   row segment (the same records the forward step uses for forces).
+// k_adj_particles : eight lanes per particle, one per corner of its cell, a
+//   vector's components one per lane (as k_particles, and for the same reason:
+//   an FP64 warp instruction takes 64 cycles whatever its lanes).  From the
+//   recorded state it gathers u(x_p), re-evaluates the particle's forward step
+//   in FP64 and runs what the chain rule needs of it through the update and
+//   the random force -- all before the launch dependency resolves, beside the
+//   lattice kernel of the reverse step before; then it gathers
+//   lam_F(x_p) = sum_a 3 w_a e_a lam_a(x_p) (the adjoint of the body-force term)
+//   and runs the chain rule back through the spreading weights and the
+//   Stokeslet fit, about 90 FP64 instructions for four particles.  What the fit
+//   sends back to the fluid is lam_u(x_p), the adjoint of the node velocity at
+//   each corner: it is appended, as (x, 3 FP64 values), to the 256-byte record
+//   of the corner's row segment (the same records the forward step uses for
+//   forces), and the segments of the next reverse step are marked for its
+//   lattice kernel.  Before, a gather kernel and an FP64 kernel with all of a
+//   particle's components in every lane took 4.3 + 13.6 us with 8 particles and
+//   47 + 87 us with 16384, and the replay copied the particle state twice a step;
+//   a reverse sweep of 200 steps at 64^3: 13.3 -> 6.6 ms with its replay (and the
+//   recording, which copied the trajectory twice a step, 4.0 -> 2.0 ms), of 20
+//   steps at 256^3: 28.5 -> 26.3 ms.
 // k_adj_lattice : the fused adjoint of collision, moments and streaming, one
 //   thread per node, one block per 128-node row segment:
 //     lam_feq_a = w lam_a
@@ -51,14 +60,13 @@
 
 namespace lbp {
 
-constexpr int APB = 32;  // particles per block (8 threads each)
-
 struct AdjPArgs {
     const void *g;           // fhat^{n-1}, storage type St, 15 planes of P
     const float *lam;        // dL/dfhat^n, FP32, 15 planes of P
     long long P, N;
     const int *prep;         // box of each particle (batches)
     const double *r, *v;     // r^n, V^n, [3][cap]
+    const double *prev_r;    // r of the next reverse step (to mark its segments), or null
     int cap, np;
     const double *fext, *inv_mass, *gamma, *radius, *sig;
     const unsigned char *pinned;
@@ -72,143 +80,97 @@ struct AdjPArgs {
     double *acc;             // [4][np]: dL/dgamma, dL/dR, dL/dM, dL/dkT (added)
     unsigned long long *rec; // records of this adjoint step
     double *fqd;             // [3][N] overflow accumulator (FP64)
-    float *ug;               // [np][8][6] scratch: u(x_p) and lam_F(x_p) per corner
+    unsigned *marks;         // the next reverse step's marks, or null
+    unsigned mark_epoch;
 };
 
-__device__ __forceinline__ int wrap_i(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+constexpr int APN = 16;              // particles per block
+constexpr int AP_T = 8 * APN + 32;   // eight threads each, and the triggering warp
 
-// Gathers (eight threads per particle): u(x_p) of the streamed f (pull) and
-// lam_F(x_p) = sum_a 3 w_a e_a lam_a(x_p) (aligned) at the eight corners, to
-// A.ug[i][p][0..2] and A.ug[i][p][3..5].
+// the sum over the three components of a value held one component per lane
+__device__ __forceinline__ double sum_over_components(double v) {
+    return from_comp(v, 0) + from_comp(v, 1) + from_comp(v, 2);
+}
+
 template <typename St, int MAXR>
-__global__ void __launch_bounds__(256) k_adj_gather(const AdjPArgs A, const RepTable<MAXR> rt) {
+__global__ void __launch_bounds__(AP_T, 3) k_adj_particles(const AdjPArgs A, const RepTable<MAXR> rt) {
+    if (threadIdx.x >= 8 * APN) {
+        // lets this reverse step's lattice kernel launch as soon as the one before
+        // is complete (see k_particles)
+        grid_dependency_wait();
+        grid_dependents_launch();
+        return;
+    }
     const typename St::T *G = static_cast<const typename St::T *>(A.g);
-    __shared__ int s_base[APB][3];
-    const int t = threadIdx.x, lane = t & 31;
-    const int i0 = blockIdx.x * APB;
-    const int cap = A.cap;
-    const int ip = i0 + lane;
-    if (t < 32 && ip < A.np) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) s_base[lane][k] = (int)floor(A.r[k * cap + ip]);
-    }
-    __syncthreads();
-
-    // ---- gathers: u(x_p) of the streamed f (pull) and lam_F(x_p) (aligned)
-    const int j = t >> 3, p = t & 7;
-    const int ij = i0 + j;
-    int X = 0, Y = 0, Z = 0;
-    const Rep &rj = rt.rep[MAXR == 1 || ij >= A.np ? 0 : A.prep[ij]];
-    const int nx = rj.nx, ny = rj.ny, nz = rj.nz;
-    const long long off = rj.node_off;
-    if (ij < A.np) {
-        X = wrap_i(s_base[j][0] + (p & 1), nx);
-        Y = wrap_i(s_base[j][1] + ((p >> 1) & 1), ny);
-        Z = wrap_i(s_base[j][2] + ((p >> 2) & 1), nz);
-        const int xs[3] = {wrap_i(X + 1, nx), X, wrap_i(X - 1, nx)};
-        const int ys[3] = {wrap_i(Y + 1, ny), Y, wrap_i(Y - 1, ny)};
-        const int zs[3] = {wrap_i(Z + 1, nz), Z, wrap_i(Z - 1, nz)};
-        float sx = 0.f, sy = 0.f, sz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
-#pragma unroll
-        for (int a = 1; a < Q; ++a) {
-            const long long src = (long long)a * A.P + off + ((long long)zs[ez(a) + 1] * ny + ys[ey(a) + 1]) * nx +
-                                  xs[ex(a) + 1];
-            const float gv = St::load(G + src, a);
-            // dL/dfhat_a(x_p) = dL/df^{n+1}_a(x_p + e_a) (the buffer's layout)
-            const long long lnode = off + ((long long)zs[1 - ez(a)] * ny + ys[1 - ey(a)]) * nx + xs[1 - ex(a)];
-            const float lv = (3.f * wgtf(a)) * __ldg(A.lam + (long long)a * A.P + lnode);
-            if (ex(a)) { sx += ex(a) > 0 ? gv : -gv; lx += ex(a) > 0 ? lv : -lv; }
-            if (ey(a)) { sy += ey(a) > 0 ? gv : -gv; ly += ey(a) > 0 ? lv : -lv; }
-            if (ez(a)) { sz += ez(a) > 0 ? gv : -gv; lz += ez(a) > 0 ? lv : -lv; }
-        }
-        float *o = A.ug + ((size_t)ij * 8 + p) * 6;
-        o[0] = sx;
-        o[1] = sy;
-        o[2] = sz;
-        o[3] = lx;
-        o[4] = ly;
-        o[5] = lz;
-    }
-}
-
-// Sum over the eight lanes of a particle (an aligned group of 8 lanes): every
-// lane gets the same value (the butterfly adds the same pairs in every lane).
-__device__ __forceinline__ double grp8_sum(double v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 4);
-    return v;
-}
-
-// The FP64 adjoint of one particle's step with eight lanes per particle, one
-// per corner of its cell: the per-corner terms of the fit (its forward
-// re-evaluation and its adjoint) and of the spreading run in parallel and meet
-// in group sums, which cuts the serial FP64 chain of a particle about
-// fourfold; the per-particle scalars (the Langevin update, the random force)
-// are evaluated in every lane of the group.  Blocks of 64 threads (8
-// particles), so that many warps share the narrow FP64 pipe.  Each lane
-// appends its corner's lam_u(x_p) to the record of that corner's row segment.
-template <int MAXR>
-__global__ void __launch_bounds__(64) k_adj_fp64(const AdjPArgs A, const RepTable<MAXR> rt) {
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = (tid >> 3) < A.np;
-    const int i = valid ? tid >> 3 : A.np - 1;  // lanes past the last particle shadow it (no stores)
-    const int c = tid & 7;                      // the lane's corner: offsets (c & 1, c >> 1 & 1, c >> 2)
-    const int cap = A.cap;
-    double r[3], V[3], q[3], lV[3], lr[3], fe[3];
-    int base[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        r[k] = A.r[k * cap + i];
-        V[k] = A.v[k * cap + i];
-        base[k] = (int)floor(r[k]);
-        q[k] = r[k] - (double)base[k];
-        fe[k] = A.fext[k * cap + i];
-        lV[k] = A.lam_v[k * cap + i] + (A.gv ? A.gv[3 * i + k] : 0.0);
-        lr[k] = A.lam_r[k * cap + i] + (A.gr ? A.gr[3 * i + k] : 0.0);
-    }
+    const int p = threadIdx.x & 7, kc = comp_of(p);
+    const int ip = blockIdx.x * APN + (threadIdx.x >> 3);
+    const bool live = ip < A.np;
+    const int i = live ? ip : A.np - 1, cap = A.cap;  // lanes past the last particle shadow it (no stores)
+    const int ik = kc * cap + i;
+    const double rk = __ldcg(A.r + ik), Vk = __ldcg(A.v + ik);
+    double lV = __ldcg(A.lam_v + ik) + (A.gv ? A.gv[3 * (size_t)i + kc] : 0.0);
+    double lr = __ldcg(A.lam_r + ik) + (A.gr ? A.gr[3 * (size_t)i + kc] : 0.0);
+    const double fek = A.fext[ik];
     const double gam = A.gamma[i], R = A.radius[i], invM = A.inv_mass[i], sg = A.sig[i];
     const bool pin = A.pinned[i] != 0;
-    // this corner's gathered u(x_p) and lam_F(x_p), and its trilinear weight
-    double u[3], lF[3], Wp = 1.0;
+    const Rep &rp = rt.rep[MAXR == 1 ? 0 : A.prep[i]];
+    const int nx = rp.nx, ny = rp.ny, nz = rp.nz;
+    const double bk = floor(rk), qk = rk - bk;
+    const int base = (int)bk;
+    const int c0 = p & 1, c1 = (p >> 1) & 1, c2 = p >> 2;
+    const int X = wrapi(from_comp(base, 0) + c0, nx), Y = wrapi(from_comp(base, 1) + c1, ny),
+              Z = wrapi(from_comp(base, 2) + c2, nz);
+    const int xs[3] = {wrapi(X + 1, nx), X, wrapi(X - 1, nx)};
+    const int ys[3] = {wrapi(Y + 1, ny), Y, wrapi(Y - 1, ny)};
+    const int zs[3] = {wrapi(Z + 1, nz), Z, wrapi(Z - 1, nz)};
+    // u(x_p) of the streamed f (pull)
+    double u[3];
     {
-        const float *g = A.ug + ((size_t)i * 8 + c) * 6;
+        float s[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            u[k] = (double)g[k];
-            lF[k] = (double)g[3 + k];
-            Wp *= ((c >> k) & 1) ? q[k] : 1.0 - q[k];
+        for (int a = 1; a < Q; ++a) {
+            const float g = St::gather(G + ((long long)a * A.P + rp.node_off +
+                                            ((long long)zs[ez(a) + 1] * ny + ys[ey(a) + 1]) * nx + xs[ex(a) + 1]), a);
+            if (ex(a)) s[0] += ex(a) > 0 ? g : -g;
+            if (ey(a)) s[1] += ey(a) > 0 ? g : -g;
+            if (ez(a)) s[2] += ez(a) > 0 ? g : -g;
         }
-    }
-    double d[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) d[k] = (double)((c >> k) & 1) - q[k];
-    // forward re-evaluation of F_H
-    double FH[3] = {0.0, 0.0, 0.0}, e[3] = {0.0, 0.0, 0.0};
-    double U = 0.0, num = 0.0, den = 0.0, nw = 0.0, inw = 0.0, iden = 0.0;
-    double ur[3] = {0.0, 0.0, 0.0};
-    bool fit = false;
-    // this corner's fit geometry (used by the forward and the adjoint fit)
-    bool use = false;
-    double rp = 0.0, ir = 0.0, ir3 = 0.0, x = 0.0, k1 = 0.0, k2 = 0.0, av[3] = {0.0, 0.0, 0.0};
+        for (int k = 0; k < 3; ++k) u[k] = widen_f32(s[k]);
+    }
+    // the random force of this step (same Philox numbers as the forward step)
+    unsigned long long ctr[4] = {(unsigned long long)A.step, (unsigned long long)i, 0ull, 0ull};
+    philox4x64_10(ctr, A.seed, 0ull);
+    const unsigned long long bits = kc == 0 ? ctr[0] : kc == 1 ? ctr[1] : ctr[2];
+    const double xi =
+        __dmul_rn(A.sqrt3, __fma_rn(__ull2double_rn(2ull * (bits >> 11) + 1ull), 0x1.0p-53, -1.0));
+    const double FR = __dmul_rn(sg, xi);
+    // this corner's trilinear weight W_p and dW_p/dq_k
+    const double q0 = from_comp(qk, 0), q1 = from_comp(qk, 1), q2 = from_comp(qk, 2);
+    const double t0 = c0 ? q0 : 1.0 - q0, t1 = c1 ? q1 : 1.0 - q1, t2 = c2 ? q2 : 1.0 - q2;
+    const double t01 = t0 * t1, Wp = t01 * t2;
+    const double dw[3] = {c0 ? t1 * t2 : -(t1 * t2), c1 ? t0 * t2 : -(t0 * t2), c2 ? t01 : -t01};
+    // forward re-evaluation of F_H (component kc), with the fit's corner terms
+    const double V[3] = {from_comp(Vk, 0), from_comp(Vk, 1), from_comp(Vk, 2)};
+    double FH = 0.0, e[3] = {0.0, 0.0, 0.0}, ek = 0.0, U = 0.0, num = 0.0, inw = 0.0, iden = 0.0, urk = 0.0;
+    double d[3] = {0.0, 0.0, 0.0}, ir = 0.0, ir3 = 0.0, x = 0.0, k1 = 0.0, k2 = 0.0, av[3] = {0.0, 0.0, 0.0};
+    bool fit = false, use = false;
     const double cR = 0.75 * R;
     if (A.mode == LBP_STOKESLET) {
-        double m[3];
+        d[0] = (double)c0 - q0;
+        d[1] = (double)c1 - q1;
+        d[2] = (double)c2 - q2;
+        const double mk = (sum_components(u[0], u[1], u[2], p) - 8.0 * Vk) * 0.125;
+        const double mm = sum_over_components(mk * mk);
+        if (mm > 0.0) inw = rsqrt(mm);
+        ek = mk * inw;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) m[k] = grp8_sum(u[k] - V[k]) * 0.125;
-        // reciprocal square roots instead of square roots and divisions (the
-        // FP64 pipe is narrow and divisions are long sequences on it)
-        const double mm = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
-        if (mm > 0.0) {
-            inw = rsqrt(mm);
-            nw = mm * inw;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) e[k] = m[k] * inw;
-        }
+        for (int k = 0; k < 3; ++k) e[k] = from_comp(ek, k);
         const double rr = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
         ir = rr > 0.0 ? rsqrt(rr) : 0.0;
-        rp = rr * ir;
-        use = nw > 0.0 && !(rp < 1e-12 || (A.exclude_inside && rp < R));
+        const double dist = rr * ir;
+        const bool moving = mm > 0.0;
+        use = moving && !(dist < 1e-12 || (A.exclude_inside && dist < R));
         double pn = 0.0, pd = 0.0;
         if (use) {
             ir3 = ir * ir * ir;
@@ -222,167 +184,142 @@ __global__ void __launch_bounds__(64) k_adj_fp64(const AdjPArgs A, const RepTabl
                 pd += av[k] * av[k];
             }
         }
-        num = grp8_sum(pn);
-        den = grp8_sum(pd);
-        if (nw > 0.0 && den != 0.0) {
+        const double nd = sum_pair(pn, pd, p);
+        num = __shfl_sync(0xffffffffu, nd, 0, 8);
+        const double den = __shfl_sync(0xffffffffu, nd, 1, 8);
+        if (moving && den != 0.0) {
             iden = 1.0 / den;
             U = num * iden;
             fit = true;
         }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) FH[k] = gam * U * e[k];
+        FH = gam * U * ek;
     } else if (A.mode == LBP_POINTWISE) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            ur[k] = grp8_sum(Wp * u[k]);
-            FH[k] = -gam * (V[k] - ur[k]);
-        }
+        urk = sum_components(Wp * u[0], Wp * u[1], Wp * u[2], p);
+        FH = -gam * (Vk - urk);
     } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) FH[k] = -gam * V[k];
+        FH = -gam * Vk;
     }
-    // the random force of this step (same Philox numbers as the forward step)
-    unsigned long long ctr[4] = {(unsigned long long)A.step, (unsigned long long)i, 0ull, 0ull};
-    philox4x64_10(ctr, A.seed, 0ull);
-    double xi[3], FR[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const double tt = __fma_rn(__ull2double_rn(2ull * (ctr[k] >> 11) + 1ull), 0x1.0p-53, -1.0);
-        xi[k] = __dmul_rn(A.sqrt3, tt);
-        FR[k] = __dmul_rn(sg, xi[k]);
+    // r' = r + V'  then  V' = V + (F_H + F_R + F_ext)/M, backwards
+    double lFH = 0.0, gG = 0.0, gR = 0.0, gM = 0.0, gK = 0.0;
+    if (!pin) {
+        lV += lr;
+        lFH = lV * invM;
+    }
+    {
+        const double lFR_xi = sum_over_components(lFH * xi);
+        const double lF_tot = sum_over_components(lV * (FH + FR + fek));
+        if (!pin) {
+            gM = -lF_tot * invM * invM;
+            // F_R = sigma xi, sigma = sqrt(2 gamma kT)
+            if (sg > 0.0) {
+                const double isg = 1.0 / sg;
+                gG += lFR_xi * (A.kT * isg);
+                gK += lFR_xi * (gam * isg);
+            }
+        }
+    }
+    const double F[3] = {from_comp(FH, 0), from_comp(FH, 1), from_comp(FH, 2)};
+    if (A.marks && A.prev_r) {
+        // mark the row segment of corner p of the next reverse step's cell
+        const int b = (int)floor(__ldcg(A.prev_r + ik));
+        const int x1 = wrapi(from_comp(b, 0) + c0, nx), y1 = wrapi(from_comp(b, 1) + c1, ny),
+                  z1 = wrapi(from_comp(b, 2) + c2, nz);
+        if (live) A.marks[rp.seg_off + ((long long)z1 * ny + y1) * rp.nchunks + x1 / SEG] = A.mark_epoch;
     }
 
-    // ---- backward
-    double lFH[3] = {0.0, 0.0, 0.0}, lq[3] = {0.0, 0.0, 0.0};
-    double gG = 0.0, gR = 0.0, gM = 0.0, gK = 0.0;
-    if (!pin) {
-        // r' = r + V'  then  V' = V + (F_H + F_R + F_ext)/M
-        double lFR_xi = 0.0, lF_tot = 0.0;
+    // ---- the lattice kernel of the reverse step before is complete
+    grid_dependency_wait();
+    double lq = 0.0, lu[3] = {0.0, 0.0, 0.0};  // adjoints of q (component kc) and of u(x_p)
+    if (A.mode != LBP_BROWNIAN) {
+        // lam_F(x_p) (aligned): dL/dfhat_a(x_p) = dL/df^{n+1}_a(x_p + e_a), the buffer's layout
+        float s[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lV[k] += lr[k];
-            lFH[k] = lV[k] * invM;
-            lFR_xi += lV[k] * invM * xi[k];
-            lF_tot += lV[k] * (FH[k] + FR[k] + fe[k]);
+        for (int a = 1; a < Q; ++a) {
+            const float l = (3.f * wgtf(a)) *
+                            __ldcg(A.lam + ((long long)a * A.P + rp.node_off +
+                                            ((long long)zs[1 - ez(a)] * ny + ys[1 - ey(a)]) * nx + xs[1 - ex(a)]));
+            if (ex(a)) s[0] += ex(a) > 0 ? l : -l;
+            if (ey(a)) s[1] += ey(a) > 0 ? l : -l;
+            if (ez(a)) s[2] += ez(a) > 0 ? l : -l;
         }
-        gM = -lF_tot * invM * invM;
-        // F_R = sigma xi, sigma = sqrt(2 gamma kT)
-        if (sg > 0.0) {
-            const double isg = 1.0 / sg;
-            gG += lFR_xi * (A.kT * isg);
-            gK += lFR_xi * (gam * isg);
-        }
-    }
-    const bool spread = A.mode != LBP_BROWNIAN;
-    // dW_p/dq_k of this corner
-    double dw[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        dw[k] = ((c >> k) & 1) ? 1.0 : -1.0;
-#pragma unroll
-        for (int j2 = 0; j2 < 3; ++j2)
-            if (j2 != k) dw[k] *= ((c >> j2) & 1) ? q[j2] : 1.0 - q[j2];
-    }
-    if (spread) {
+        const double lF[3] = {widen_f32(s[0]), widen_f32(s[1]), widen_f32(s[2])};
         // F(x_p) += -F_H W_p(q)
-        const double fl = FH[0] * lF[0] + FH[1] * lF[1] + FH[2] * lF[2];
+        double fl = F[0] * lF[0] + F[1] * lF[1] + F[2] * lF[2];
+        lFH -= sum_components(Wp * lF[0], Wp * lF[1], Wp * lF[2], p);
+        const double lf[3] = {from_comp(lFH, 0), from_comp(lFH, 1), from_comp(lFH, 2)};
+        if (A.mode == LBP_STOKESLET) {
+            // the adjoint of the fit, with zero terms where there was none
+            const double eF = e[0] * lf[0] + e[1] * lf[1] + e[2] * lf[2];
+            const double lU = fit ? gam * eF : 0.0;
+            if (fit) gG += U * eF;
+            const double lnum = lU * iden, lden = -lnum * num * iden;
+            double ple[3] = {0.0, 0.0, 0.0}, plc = 0.0, pq[3] = {fl * dw[0], fl * dw[1], fl * dw[2]};
+            if (use && fit) {
+                double la[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lFH[k] -= grp8_sum(Wp * lF[k]);
-            lq[k] -= grp8_sum(fl * dw[k]);
-        }
-    }
-    double lu[3] = {0.0, 0.0, 0.0};  // this corner's lam_u(x_p)
-    if (A.mode == LBP_STOKESLET) {
-        // the adjoint of the fit, with zero terms where there was none
-        const double eF = e[0] * lFH[0] + e[1] * lFH[1] + e[2] * lFH[2];
-        const double lU = fit ? gam * eF : 0.0;
-        if (fit) gG += U * eF;
-        double le[3] = {gam * U * lFH[0], gam * U * lFH[1], gam * U * lFH[2]};
-        const double lnum = fit ? lU * iden : 0.0, lden = fit ? -lU * num * iden * iden : 0.0;
-        double ple[3] = {0.0, 0.0, 0.0}, pq[3] = {0.0, 0.0, 0.0}, plc = 0.0;
-        if (use && fit) {
-            const double ir5 = ir3 * ir * ir;
-            double la[3];
+                for (int k = 0; k < 3; ++k) {
+                    lu[k] = lnum * av[k];
+                    la[k] = lnum * (u[k] - V[k]) + 2.0 * lden * av[k];
+                }
+                const double dla = d[0] * la[0] + d[1] * la[1] + d[2] * la[2];
+                const double lk1 = e[0] * la[0] + e[1] * la[1] + e[2] * la[2];
+                const double c3 = cR * ir3;
+                const double cd = c3 * lk1 + 3.0 * dla * (k2 * (ir * ir)), ce = c3 * dla;  // of d_k and e_k below
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lu[k] += lnum * av[k];
-                la[k] = lnum * (u[k] - V[k]) + 2.0 * lden * av[k];
+                for (int k = 0; k < 3; ++k) {
+                    ple[k] = k1 * la[k] - ce * d[k];
+                    pq[k] += cd * d[k] - k2 * la[k] - ce * e[k];
+                }
+                plc = -lk1 * ir - dla * x * ir3;
             }
-            const double dla = d[0] * la[0] + d[1] * la[1] + d[2] * la[2];
-            const double lk1 = e[0] * la[0] + e[1] * la[1] + e[2] * la[2];
-            const double lk2 = -dla;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                ple[k] = k1 * la[k] - cR * ir3 * d[k] * dla;
-                pq[k] = -k2 * la[k] + lk1 * cR * ir3 * d[k] + lk2 * cR * (ir3 * e[k] - 3.0 * x * ir5 * d[k]);
-            }
-            plc = -lk1 * ir + lk2 * x * ir3;
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            le[k] += grp8_sum(ple[k]);
-            lq[k] -= grp8_sum(pq[k]);
-        }
-        const double lc = grp8_sum(plc);
-        if (fit) {
-            gR += 0.75 * lc;
+            const double le = gam * U * lFH + sum_components(ple[0], ple[1], ple[2], p);
+            lq = -sum_components(pq[0], pq[1], pq[2], p);
+            const double lc = sum_pair(plc, 0.0, p);  // in even lanes
+            if (fit) gR += 0.75 * lc;
             // e = m/|m| with m the mean of the w_p
-            const double ee = e[0] * le[0] + e[1] * le[1] + e[2] * le[2];
+            const double ee = sum_over_components(ek * le);
+            const double lm = fit ? (le - ek * ee) * (inw * 0.125) : 0.0;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) lu[k] += (le[k] - e[k] * ee) * inw * 0.125;
-        }
-        // w_p = u_p - V
+            for (int k = 0; k < 3; ++k) lu[k] += from_comp(lm, k);
+            // w_p = u_p - V
+            lV -= sum_components(lu[0], lu[1], lu[2], p);
+        } else {
+            gG += -sum_over_components((Vk - urk) * lFH);
+            const double ul = gam * (u[0] * lf[0] + u[1] * lf[1] + u[2] * lf[2]);
+            fl -= ul;
+            lq = -sum_components(fl * dw[0], fl * dw[1], fl * dw[2], p);
+            lV -= gam * lFH;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) lV[k] -= grp8_sum(lu[k]);
-    } else if (A.mode == LBP_POINTWISE) {
-        gG += -((V[0] - ur[0]) * lFH[0] + (V[1] - ur[1]) * lFH[1] + (V[2] - ur[2]) * lFH[2]);
-        const double ul = u[0] * lFH[0] + u[1] * lFH[1] + u[2] * lFH[2];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lV[k] -= gam * lFH[k];
-            lu[k] = gam * Wp * lFH[k];
-            lq[k] += grp8_sum(gam * ul * dw[k]);
+            for (int k = 0; k < 3; ++k) lu[k] = gam * Wp * lf[k];
         }
     } else {
-        gG += -(V[0] * lFH[0] + V[1] * lFH[1] + V[2] * lFH[2]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) lV[k] -= gam * lFH[k];
+        gG += -sum_over_components(Vk * lFH);
+        lV -= gam * lFH;
     }
-    if (!valid) return;  // past the shuffles: shadow lanes leave
-    if (c == 0) {
-        // q = r - floor(r)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lr[k] += lq[k];
-            A.lam_v[k * cap + i] = lV[k];
-            A.lam_r[k * cap + i] = lr[k];
-        }
-        A.acc[i] += gG;
-        A.acc[A.np + i] += gR;
-        A.acc[2 * A.np + i] += gM;
-        A.acc[3 * A.np + i] += gK;
+    if (!live) return;  // past the shuffles
+    if (p < 3) {
+        A.lam_v[ik] = lV;
+        A.lam_r[ik] = lr + lq;  // q = r - floor(r)
+    }
+    // gG and gK are in every lane, gR in the even ones
+    if (p < 4) {
+        double *acc = A.acc + (size_t)(p == 2 ? 1 : p == 1 ? 2 : p) * A.np + i;
+        *acc = __ldcg(acc) + (p == 0 ? gG : p == 1 ? gM : p == 2 ? gR : gK);
     }
     // lam_u(x_p) of this corner to the record of its row segment
-    if (spread && !(lu[0] == 0.0 && lu[1] == 0.0 && lu[2] == 0.0)) {
-        const Rep &ri = rt.rep[MAXR == 1 ? 0 : A.prep[i]];
-        const int nx = ri.nx, ny = ri.ny, nz = ri.nz;
-        const int X = wrap_i(base[0] + (c & 1), nx);
-        const int Y = wrap_i(base[1] + ((c >> 1) & 1), ny);
-        const int Z = wrap_i(base[2] + ((c >> 2) & 1), nz);
+    if (A.mode != LBP_BROWNIAN && !(lu[0] == 0.0 && lu[1] == 0.0 && lu[2] == 0.0)) {
         const long long row = (long long)Z * ny + Y;
-        unsigned long long *rec = A.rec + (size_t)(ri.seg_off + row * ri.nchunks + X / SEG) * REC_WORDS;
+        unsigned long long *rec = A.rec + (size_t)(rp.seg_off + row * rp.nchunks + X / SEG) * REC_WORDS;
         const unsigned int slot = atomicAdd(reinterpret_cast<unsigned int *>(rec), 1u);
         if (slot < (unsigned)REC_SLOTS) {
             reinterpret_cast<int *>(rec + REC_X0)[slot] = X;
-            rec[REC_F0 + 3 * slot] = (unsigned long long)__double_as_longlong(lu[0]);
-            rec[REC_F0 + 3 * slot + 1] = (unsigned long long)__double_as_longlong(lu[1]);
-            rec[REC_F0 + 3 * slot + 2] = (unsigned long long)__double_as_longlong(lu[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                rec[REC_F0 + 3 * slot + k] = (unsigned long long)__double_as_longlong(lu[k]);
         } else {
-            const long long node = ri.node_off + row * nx + X;
-            atomicAdd(A.fqd + node, lu[0]);
-            atomicAdd(A.fqd + A.N + node, lu[1]);
-            atomicAdd(A.fqd + 2 * A.N + node, lu[2]);
+            const long long node = rp.node_off + row * nx + X;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) atomicAdd(A.fqd + k * A.N + node, lu[k]);
         }
     }
 }
@@ -396,8 +333,8 @@ __device__ __forceinline__ void adj_record_sum(const unsigned long long *rec, un
         unsigned long long b0 = 0, b1 = 0, b2 = 0;
         for (unsigned m = mask; m; m &= m - 1) {
             const int sl = __ffs(m) - 1;
-            const unsigned long long v0 = rec[REC_F0 + 3 * sl], v1 = rec[REC_F0 + 3 * sl + 1],
-                                     v2 = rec[REC_F0 + 3 * sl + 2];
+            const unsigned long long v0 = __ldcg(rec + REC_F0 + 3 * sl), v1 = __ldcg(rec + REC_F0 + 3 * sl + 1),
+                                     v2 = __ldcg(rec + REC_F0 + 3 * sl + 2);
             if (best < 0 || v0 < b0 || (v0 == b0 && (v1 < b1 || (v1 == b1 && v2 < b2)))) {
                 best = sl;
                 b0 = v0;
@@ -416,11 +353,11 @@ __device__ __forceinline__ void adj_record_sum(const unsigned long long *rec, un
 // measured 6.5% faster at 256^3 (more bytes in flight per SM).
 template <typename St, int MAXR>
 __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__restrict__ G,
-                                                     const float *__restrict__ lam, float *lam_out,
+                                                     const float *lam, float *lam_out,
                                                      long long P, const RepTable<MAXR> rt,
                                                      const unsigned long long *rec_cur,
                                                      unsigned long long *rec_prev, double *fqd,
-                                                     long long N, double *acc_omega) {
+                                                     long long N, double *acc_omega, const Marks mk) {
     __shared__ float s_red[SEG / 32];
     // the block's box (batches: one block per row segment of every box, in box order)
     const int rb = find_block_rep(rt, blockIdx.x);
@@ -448,11 +385,16 @@ __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__
     for (int a = 0; a < Q; ++a) {
         const int o = ox[ex(a) + 1] + oy[ey(a) + 1] + oz[ez(a) + 1];   // x - e_a
         const int op = ox[1 - ex(a)] + oy[1 - ey(a)] + oz[1 - ez(a)];  // x + e_a
-        g[a] = St::load(G + (long long)a * P + d + o, a);
+        g[a] = St::gather(G + (long long)a * P + d + o, a);
         // dL/dfhat^n_a(x) = dL/df^{n+1}_a(x + e_a): the buffer holds the latter
-        l[a] = __ldg(lam + (long long)a * P + d + op);
+        l[a] = __ldcg(lam + (long long)a * P + d + op);
     }
-    const unsigned long long rw = __ldg(rec_cur + seg * REC_WORDS + lane);
+    // the records come from this reverse step's particle kernel: only marked
+    // segments wait for it (and block 0, so that this grid never ends before it)
+    const bool marked = mk.epoch == 0 || __ldcg(mk.seg + seg) == mk.epoch;
+    if (marked || blockIdx.x == 0) grid_dependency_wait();
+    grid_dependents_launch();
+    const unsigned long long rw = marked ? __ldcg(rec_cur + seg * REC_WORDS + lane) : 0ull;
     // particle contributions lam_u(x)
     float pu0 = 0.f, pu1 = 0.f, pu2 = 0.f;
     const int cnt = (int)(unsigned)(__shfl_sync(0xffffffffu, rw, 0) & 0xffffffffull);
@@ -467,9 +409,9 @@ __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__
         if (mask && act)
             adj_record_sum(rec_cur + seg * REC_WORDS, mask, a0, a1, a2);
         if (cnt > REC_SLOTS && act) {
-            a0 += fqd[d];
-            a1 += fqd[N + d];
-            a2 += fqd[2 * N + d];
+            a0 += __ldcg(fqd + d);
+            a1 += __ldcg(fqd + N + d);
+            a2 += __ldcg(fqd + 2 * N + d);
             fqd[d] = 0.0;
             fqd[N + d] = 0.0;
             fqd[2 * N + d] = 0.0;
@@ -536,7 +478,7 @@ __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < SEG / 32; ++w) s += s_red[w];
-        acc_omega[blockIdx.x] += (double)s;
+        acc_omega[blockIdx.x] = __ldcg(acc_omega + blockIdx.x) + (double)s;
     }
 }
 
@@ -574,19 +516,17 @@ static cudaError_t by_batch_adj(const Sim &s, F &&f) {
     return f(adj_table<MAX_BATCH>(s));
 }
 
-cudaError_t launch_adj_particles(Sim &s, const void *g, const float *lam, const double *r,
-                                 const double *v, long long step, const double *gv,
-                                 const double *gr, double *lam_v, double *lam_r, double *acc,
-                                 int parity, float *ug, cudaStream_t st) {
+cudaError_t launch_adj_particles(Sim &s, const AdjStep &a, cudaStream_t st, bool chained) {
     if (s.np == 0) return cudaSuccess;
     AdjPArgs A;
-    A.g = g;
-    A.lam = lam;
+    A.g = a.g;
+    A.lam = a.lam;
     A.P = s.P;
     A.N = s.N;
     A.prep = s.prep;
-    A.r = r;
-    A.v = v;
+    A.r = a.state;
+    A.v = a.state + 3 * (size_t)s.cap;
+    A.prev_r = a.prev_state;
     A.cap = s.cap;
     A.np = s.np;
     A.fext = s.fext;
@@ -597,46 +537,46 @@ cudaError_t launch_adj_particles(Sim &s, const void *g, const float *lam, const 
     A.pinned = s.pinned;
     A.kT = s.kT;
     A.seed = s.seed;
-    A.step = step;
+    A.step = a.step;
     A.sqrt3 = s.sqrt3;
     A.mode = s.mode;
     A.exclude_inside = s.exclude_inside;
-    A.gv = gv;
-    A.gr = gr;
-    A.lam_v = lam_v;
-    A.lam_r = lam_r;
-    A.acc = acc;
-    A.rec = s.rec[parity];
+    A.gv = a.gv;
+    A.gr = a.gr;
+    A.lam_v = a.lam_v;
+    A.lam_r = a.lam_r;
+    A.acc = a.acc;
+    A.rec = s.rec[a.parity];
     A.fqd = reinterpret_cast<double *>(s.fq);
-    A.ug = ug;
-    const unsigned grid = (unsigned)((s.np + APB - 1) / APB);
-    return by_batch_adj(s, [&](const auto &rt) {
-        constexpr int MAXR = sizeof(rt.rep) / sizeof(Rep);
-        cudaError_t e = by_storage_adj(s.precision, [&](auto tag) {
-            using St = decltype(tag);
-            k_adj_gather<St, MAXR><<<grid, 8 * APB, 0, st>>>(A, rt);
-            return cudaGetLastError();
-        });
-        if (e != cudaSuccess) return e;
-        k_adj_fp64<MAXR><<<(unsigned)((8 * s.np + 63) / 64), 64, 0, st>>>(A, rt);
-        return cudaGetLastError();
-    });
-}
-
-cudaError_t launch_adj_lattice(Sim &s, const void *g, const float *lam, float *lam_out, int parity,
-                               double *acc_omega, cudaStream_t st) {
-    const unsigned grid = (unsigned)adj_lattice_blocks(s);
+    A.marks = a.next && s.mode != LBP_BROWNIAN ? s.marks[a.next & 1] : nullptr;
+    A.mark_epoch = a.next;
+    const unsigned grid = (unsigned)((s.np + APN - 1) / APN);
     return by_batch_adj(s, [&](const auto &rt) {
         constexpr int MAXR = sizeof(rt.rep) / sizeof(Rep);
         return by_storage_adj(s.precision, [&](auto tag) {
             using St = decltype(tag);
-            k_adj_lattice<St, MAXR><<<grid, SEG, 0, st>>>(static_cast<const typename St::T *>(g), lam, lam_out,
-                                                          s.P, rt, s.rec[parity], s.rec[parity ^ 1],
-                                                          reinterpret_cast<double *>(s.fq), s.N, acc_omega);
-            return cudaGetLastError();
+            return launch_k(k_adj_particles<St, MAXR>, grid, AP_T, 0, st, chained, A, rt);
         });
     });
 }
+
+cudaError_t launch_adj_lattice(Sim &s, const AdjStep &a, cudaStream_t st, bool pdl) {
+    const unsigned grid = (unsigned)adj_lattice_blocks(s);
+    const Marks mk{s.marks[a.epoch & 1], a.epoch};
+    return by_batch_adj(s, [&](const auto &rt) {
+        constexpr int MAXR = sizeof(rt.rep) / sizeof(Rep);
+        return by_storage_adj(s.precision, [&](auto tag) {
+            using St = decltype(tag);
+            const unsigned long long *rec = s.rec[a.parity];
+            return launch_k(k_adj_lattice<St, MAXR>, grid, SEG, 0, st, pdl, static_cast<const typename St::T *>(a.g),
+                            a.lam, a.lam_out, (long long)s.P, rt, rec, s.rec[a.parity ^ 1],
+                            reinterpret_cast<double *>(s.fq), (long long)s.N, a.acc_omega, mk);
+        });
+    });
+}
+
+// Marks pay where the lattice kernel's blocks are more than are resident (six per SM).
+bool adj_lattice_marks(const Sim &s) { return s.np > 0 && adj_lattice_blocks(s) > 6 * s.num_sms; }
 
 int adj_lattice_blocks(const Sim &s) {
     int n = 0;

@@ -1257,6 +1257,7 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     for (int64_t n = 0; n < nsteps; ++n) {
         if (n % checkpoint_every == 0) {
             const int64_t k = n / checkpoint_every;
+            c.follows = false;  // copies follow the last step
             CK(cudaMemcpyAsync(tp.ck_f + (size_t)k * pop_bytes, s->f[s->cur], pop_bytes,
                                cudaMemcpyDeviceToDevice, s->s0));
             if (s->np > 0) {
@@ -1266,10 +1267,10 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
                                    sizeof(double) * 3 * s->cap, cudaMemcpyDeviceToDevice, s->s0));
             }
         }
-        c.follows = false;  // copies were queued since the last step
-        TRY(step_once(s, c));
-        if (vt) CK(launch_soa_to_aos(s->v, vt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
-        if (rt) CK(launch_soa_to_aos(s->r, rt + (size_t)n * s->np * 3, s->np, s->cap, s->s0));
+        // the particle kernel writes the trajectories itself
+        const ParticleIO io{nullptr, rt ? rt + (size_t)n * s->np * 3 : nullptr, vt ? vt + (size_t)n * s->np * 3 : nullptr,
+                            false};
+        TRY(step_once(s, c, &io));
     }
     if (!on_device && traj > 0) {
         if (v_traj) CK(cudaMemcpyAsync(v_traj, vt, sizeof(double) * traj, cudaMemcpyDeviceToHost, s->s0));
@@ -1316,16 +1317,13 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
     guard.p.push_back(seg);
     TRY(dalloc(&lam, (size_t)2 * Q * s->P));
     guard.p.push_back(lam);
-    float *ug = nullptr;  // per-corner gathers of the particle adjoint
-    TRY(dalloc(&ug, (size_t)48 * (np > 0 ? np : 1)));
-    guard.p.push_back(ug);
     // doubles: seg_p [C][6 cap] | lam_v, lam_r [3 cap] | acc [4 np] | acc_om [nblk] |
-    //          save (r, v, fh, fr) [12 cap] | g_v, g_r staged [traj] each
+    //          g_v, g_r staged [traj] each
     const size_t n_segp = (size_t)C * pcount, n_lvr = (size_t)6 * cap, n_acc = (size_t)4 * (np > 0 ? np : 1),
-                 n_om = (size_t)nblk, n_save = (size_t)12 * cap;
+                 n_om = (size_t)nblk;
     const bool stage_g = !on_device && traj > 0;
     const size_t n_g = stage_g ? 2 * traj : 0;
-    TRY(dalloc(&dwork, n_segp + n_lvr + n_acc + n_om + n_save + n_g));
+    TRY(dalloc(&dwork, n_segp + n_lvr + n_acc + n_om + n_g));
     guard.p.push_back(dwork);
     double *f0tmp = nullptr;  // FP64 staging of dL/df0 for a host destination
     if (out->f0 && !on_device) {
@@ -1333,7 +1331,7 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
         guard.p.push_back(f0tmp);
     }
     double *seg_p = dwork, *lam_v = seg_p + n_segp, *lam_r = lam_v + 3 * (size_t)cap,
-           *acc = lam_v + n_lvr, *acc_om = acc + n_acc, *save = acc_om + n_om, *gst = save + n_save;
+           *acc = lam_v + n_lvr, *acc_om = acc + n_acc, *gst = acc_om + n_om;
     const double *gv = g_v, *gr = g_r;
     if (stage_g) {
         if (g_v) {
@@ -1347,20 +1345,10 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
     }
     CK(cudaMemsetAsync(lam, 0, sizeof(float) * 2 * Q * s->P, s->s0));
     CK(cudaMemsetAsync(lam_v, 0, sizeof(double) * (n_lvr + n_acc + n_om), s->s0));
-    // the state to put back: particles (the populations are not touched)
-    double *sv[4] = {s->r, s->v, s->fh, s->fr};
-    if (np > 0)
-        for (int k = 0; k < 4; ++k)
-            CK(cudaMemcpyAsync(save + (size_t)3 * cap * k, sv[k], sizeof(double) * 3 * cap,
-                               cudaMemcpyDeviceToDevice, s->s0));
     const int saved_vacf = s->vacf_lag;
     s->vacf_lag = -1;  // the replay writes no VACF samples
     auto restore = [&]() {
         s->vacf_lag = saved_vacf;
-        if (np > 0)
-            for (int k = 0; k < 4; ++k)
-                cudaMemcpyAsync(sv[k], save + (size_t)3 * cap * k, sizeof(double) * 3 * cap,
-                                cudaMemcpyDeviceToDevice, s->s0);
         if (s->rec[0]) {
             cudaMemsetAsync(s->rec[0], 0, rec_bytes, s->s0);
             cudaMemsetAsync(s->rec[1], 0, rec_bytes, s->s0);
@@ -1382,57 +1370,57 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
         // state j of the segment: the checkpoint for j = 0, else replay slot j - 1
         char *ck = tp.ck_f + (size_t)k * pop_bytes;
         auto state = [&](int j) -> char * { return j == 0 ? ck : seg + (size_t)(j - 1) * pop_bytes; };
-        if (np > 0) {
-            ADJ_CK(cudaMemcpyAsync(s->r, tp.ck_p + (size_t)k * pcount, sizeof(double) * 3 * cap,
-                                   cudaMemcpyDeviceToDevice, s->s0));
-            ADJ_CK(cudaMemcpyAsync(s->v, tp.ck_p + (size_t)k * pcount + 3 * cap, sizeof(double) * 3 * cap,
-                                   cudaMemcpyDeviceToDevice, s->s0));
-        }
+        // the particle state of j, likewise
+        auto pstate = [&](int j) -> double * {
+            return j == 0 ? tp.ck_p + (size_t)k * pcount : seg_p + (size_t)(j - 1) * pcount;
+        };
         long long st0 = tp.step0 + n0;
         ADJ_CK(cudaMemcpyAsync(s->d_step, &st0, sizeof(long long), cudaMemcpyHostToDevice, s->s0));
         if (s->rec[0]) {
             ADJ_CK(cudaMemsetAsync(s->rec[0], 0, rec_bytes, s->s0));
             ADJ_CK(cudaMemsetAsync(s->rec[1], 0, rec_bytes, s->s0));
         }
-        for (int j = 0; j < m && e == cudaSuccess; ++j) {
-            const int64_t n = n0 + j;
-            const int parity = tp.cur0 ^ (int)(n & 1);
-            if (np > 0) {
-                ADJ_CK(cudaMemcpyAsync(seg_p + (size_t)j * pcount, s->r, sizeof(double) * 3 * cap,
-                                       cudaMemcpyDeviceToDevice, s->s0));
-                ADJ_CK(cudaMemcpyAsync(seg_p + (size_t)j * pcount + 3 * cap, s->v, sizeof(double) * 3 * cap,
-                                       cudaMemcpyDeviceToDevice, s->s0));
-            }
-            if (j == m - 1) break;
-            const void *src = state(j);
-            void *dst = state(j + 1);
-            if (np > 0) {
-                ADJ_CK(launch_particles(*s, src, parity, s->s0));
-                ADJ_CK(launch_stream_collide_forced(*s, src, dst, parity, s->s0, false));
-            } else {
-                ADJ_CK(launch_stream_collide(*s, src, dst, s->s0));
-            }
+        unsigned epoch = 0;
+        for (int j = 0; j < m - 1 && e == cudaSuccess; ++j) {
+            const int parity = tp.cur0 ^ (int)((n0 + j) & 1);
+            const unsigned next = j < m - 2 && s->chain && lattice_marks(*s) ? ++s->epoch : 0;
+            const ParticleIO io{nullptr, nullptr, nullptr, false, pstate(j), pstate(j + 1)};
+            ADJ_CK(launch_particles(*s, state(j), parity, s->s0, &io, j > 0 && s->chain && lattice_chains(*s), next));
+            ADJ_CK(launch_stream_collide_forced(*s, state(j), state(j + 1), parity, s->s0, true, epoch));
+            epoch = next;
         }
         if (s->rec[0]) {
             ADJ_CK(cudaMemsetAsync(s->rec[0], 0, rec_bytes, s->s0));
             ADJ_CK(cudaMemsetAsync(s->rec[1], 0, rec_bytes, s->s0));
         }
         // step the adjoint back through the segment
+        epoch = 0;
         for (int j = m - 1; j >= 0 && e == cudaSuccess; --j) {
             const int64_t n = n0 + j;
-            const int q = j & 1;
-            const void *src = state(j);
-            const float *lc = lam + (size_t)L * Q * s->P;
-            float *ln = lam + (size_t)(L ^ 1) * Q * s->P;
-            const double *rj = seg_p + (size_t)j * pcount, *vj = rj + 3 * cap;
-            ADJ_CK(launch_adj_particles(*s, src, lc, rj, vj, tp.step0 + n, gv ? gv + (size_t)n * np * 3 : nullptr,
-                                        gr ? gr + (size_t)n * np * 3 : nullptr, lam_v, lam_r, acc, q, ug, s->s0));
+            AdjStep a;
+            a.g = state(j);
+            a.state = pstate(j);
+            a.prev_state = j > 0 ? pstate(j - 1) : nullptr;
+            a.step = tp.step0 + n;
+            a.gv = gv ? gv + (size_t)n * np * 3 : nullptr;
+            a.gr = gr ? gr + (size_t)n * np * 3 : nullptr;
+            a.lam_v = lam_v;
+            a.lam_r = lam_r;
+            a.acc = acc;
+            a.lam = lam + (size_t)L * Q * s->P;
+            a.lam_out = lam + (size_t)(L ^ 1) * Q * s->P;
+            a.acc_omega = acc_om;
+            a.parity = j & 1;
+            a.epoch = epoch;
+            a.next = j > 0 && s->chain && adj_lattice_marks(*s) ? ++s->epoch : 0;
+            epoch = a.next;
             const bool timed = s->timing && e == cudaSuccess;
+            ADJ_CK(launch_adj_particles(*s, a, s->s0, j < m - 1 && !timed && s->chain));
             if (timed) {
                 if (s->ntimed == lbp::Sim::MAX_TIMED && fold_timing(s) != LBP_OK) e = cudaErrorUnknown;
                 ADJ_CK(cudaEventRecord(s->tev[2 * s->ntimed], s->s0));
             }
-            ADJ_CK(launch_adj_lattice(*s, src, lc, ln, q, acc_om, s->s0));
+            ADJ_CK(launch_adj_lattice(*s, a, s->s0, !timed));
             if (timed) {
                 ADJ_CK(cudaEventRecord(s->tev[2 * s->ntimed + 1], s->s0));
                 if (e == cudaSuccess) s->ntimed += 1;

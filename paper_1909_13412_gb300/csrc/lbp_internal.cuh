@@ -330,6 +330,56 @@ __device__ __forceinline__ void philox4x64_10(unsigned long long c[4], unsigned 
     }
 }
 
+// ------------------------------------------------------------ particle lanes
+// The particle kernels serve a particle with eight lanes, one per corner of its
+// cell, and keep vectors one component per lane (particle_kernels.cu).
+__device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
+
+// Component of the vectors that lane p of a particle holds, and the first lane
+// holding component k.
+__device__ __forceinline__ int comp_of(int p) { return (p & 1) ? 2 : (p >> 1) & 1; }
+__device__ __forceinline__ int lane_of(int k) { return k == 0 ? 0 : 3 - k; }
+
+// |v| < bound for bound > 0 (false for a NaN), on the bits
+__device__ __forceinline__ bool below(double v, double bound) {
+    return (__double_as_longlong(v) & 0x7fffffffffffffffll) < __double_as_longlong(bound);
+}
+
+// v < 0 (not for -0; also for a NaN with its sign set), on the bits
+__device__ __forceinline__ bool negative(double v) {
+    return (unsigned long long)__double_as_longlong(v) > 0x8000000000000000ull;
+}
+
+template <typename T>
+__device__ __forceinline__ T from_comp(T v, int k) {
+    return __shfl_sync(0xffffffffu, v, lane_of(k), 8);
+}
+
+// Sums over a particle's eight corners follow the tree
+// ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), every operation rounded explicitly.
+//
+// The sum of (v0, v1, v2), component comp_of(p) in lane p: lanes that differ in
+// the first bit split component 2 from the others, those that differ in the
+// second 0 from 1.
+__device__ __forceinline__ double sum_components(double v0, double v1, double v2, int p) {
+    const bool odd = p & 1;
+    double a = __shfl_xor_sync(0xffffffffu, odd ? v0 : v2, 1), b = __shfl_xor_sync(0xffffffffu, v1, 1);
+    a = __dadd_rn(odd ? v2 : v0, a);
+    b = __dadd_rn(v1, b);
+    const bool one = !odd && (p & 2);
+    const double c = __shfl_xor_sync(0xffffffffu, odd || one ? a : b, 2);
+    a = __dadd_rn(one ? b : a, c);
+    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
+}
+
+// the sums of x (left in even lanes) and y (in odd lanes)
+__device__ __forceinline__ double sum_pair(double x, double y, int p) {
+    const bool odd = p & 1;
+    double a = __dadd_rn(odd ? y : x, __shfl_xor_sync(0xffffffffu, odd ? x : y, 1));
+    a = __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 2));
+    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
+}
+
 // ------------------------------------------------------------ replicas
 // A handle holds one or more independent periodic boxes ("replicas", the
 // batched ensemble).  Their populations are concatenated node-wise in the same
@@ -565,6 +615,10 @@ struct ParticleIO {
     const double *fext_in;
     double *r_out, *v_out;
     bool signal;
+    // the adjoint's replay: the particle state is read from and written to these
+    // ([6][cap]: r, V) instead of the handle's arrays, and F_H, F_R are not kept
+    const double *state_in = nullptr;
+    double *state_out = nullptr;
 };
 // chained: launched right after the previous step's lattice pass on `st`, as its
 // programmatic dependent.  mark_epoch: mark the segments of the next step with
@@ -590,13 +644,27 @@ constexpr int STAGED_NODES = 512;     // nodes per item (whole rows) of the stag
 constexpr int STAGED_RECS = 16;       // force records per item of the staged kernel
 constexpr int STAGED_THREADS = 256;
 // adjoint_kernels.cu
-cudaError_t launch_adj_particles(Sim &s, const void *g, const float *lam, const double *r,
-                                 const double *v, long long step, const double *gv,
-                                 const double *gr, double *lam_v, double *lam_r, double *acc,
-                                 int parity, float *ug, cudaStream_t st);
-cudaError_t launch_adj_lattice(Sim &s, const void *g, const float *lam, float *lam_out, int parity,
-                               double *acc_omega, cudaStream_t st);
+// One reverse step, n: the state it differentiates and the adjoints it moves.
+struct AdjStep {
+    const void *g;             // populations fhat^{n-1}
+    const double *state;       // r^n, V^n ([6][cap])
+    const double *prev_state;  // those of the reverse step that follows in the chain, or null
+    long long step;            // Philox counter of step n
+    const double *gv, *gr;     // dL/dV^{n+1}, dL/dr^{n+1} ([np][3]), or null
+    double *lam_v, *lam_r;     // adjoints of the particle state ([3][cap] each)
+    double *acc;               // [4][np]: dL/dgamma, dL/dR, dL/dM, dL/dkT
+    const float *lam;          // dL/df^{n+1}
+    float *lam_out;            // dL/df^n
+    double *acc_omega;         // [adj_lattice_blocks]
+    int parity;                // of the force records
+    unsigned epoch, next;      // marks of this reverse step (0: none), and to write for the next
+};
+// chained: launched right after the previous reverse step's lattice kernel; pdl:
+// right after the particle kernel
+cudaError_t launch_adj_particles(Sim &s, const AdjStep &a, cudaStream_t st, bool chained);
+cudaError_t launch_adj_lattice(Sim &s, const AdjStep &a, cudaStream_t st, bool pdl);
 int adj_lattice_blocks(const Sim &s);
+bool adj_lattice_marks(const Sim &s);  // the reverse sweep's lattice kernel gains from marks
 int adj_lattice_first_block(const Sim &s, int replica);  // first block of a box in the adjoint lattice launch
 cudaError_t launch_f32_to_f64(Sim &s, const float *src, double *dst, cudaStream_t st);
 // vacf_kernels.cu

@@ -82,7 +82,9 @@ struct ParticleArgs {
     const int *prep; // replica (box) of each particle
     long long P;
     long long N;
-    double *r, *v, *fh, *fr;
+    const double *r_in, *v_in;  // the state to advance, and where it goes (the same, but for a replay)
+    double *r, *v;
+    double *fh, *fr;            // null in a replay
     double *fext;  // written only when fext_in is given (lbp_step_exchange)
     const double *inv_mass, *gamma, *radius, *sig;
     const unsigned char *pinned;
@@ -117,53 +119,6 @@ struct ParticleArgs {
     unsigned *done_ticket;
     long long *done_flag;
 };
-
-__device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
-
-// Component of the vectors that lane p of a particle holds, and the first lane
-// holding component k.
-__device__ __forceinline__ int comp_of(int p) { return (p & 1) ? 2 : (p >> 1) & 1; }
-__device__ __forceinline__ int lane_of(int k) { return k == 0 ? 0 : 3 - k; }
-
-// |v| < bound for bound > 0 (false for a NaN), on the bits
-__device__ __forceinline__ bool below(double v, double bound) {
-    return (__double_as_longlong(v) & 0x7fffffffffffffffll) < __double_as_longlong(bound);
-}
-
-// v < 0 (not for -0; also for a NaN with its sign set), on the bits
-__device__ __forceinline__ bool negative(double v) {
-    return (unsigned long long)__double_as_longlong(v) > 0x8000000000000000ull;
-}
-
-template <typename T>
-__device__ __forceinline__ T from_comp(T v, int k) {
-    return __shfl_sync(0xffffffffu, v, lane_of(k), 8);
-}
-
-// Sums over a particle's eight corners follow the tree
-// ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), every operation rounded explicitly.
-//
-// The sum of (v0, v1, v2), component comp_of(p) in lane p: lanes that differ in
-// the first bit split component 2 from the others, those that differ in the
-// second 0 from 1.
-__device__ __forceinline__ double sum_components(double v0, double v1, double v2, int p) {
-    const bool odd = p & 1;
-    double a = __shfl_xor_sync(0xffffffffu, odd ? v0 : v2, 1), b = __shfl_xor_sync(0xffffffffu, v1, 1);
-    a = __dadd_rn(odd ? v2 : v0, a);
-    b = __dadd_rn(v1, b);
-    const bool one = !odd && (p & 2);
-    const double c = __shfl_xor_sync(0xffffffffu, odd || one ? a : b, 2);
-    a = __dadd_rn(one ? b : a, c);
-    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
-}
-
-// the sums of x (left in even lanes) and y (in odd lanes)
-__device__ __forceinline__ double sum_pair(double x, double y, int p) {
-    const bool odd = p & 1;
-    double a = __dadd_rn(odd ? y : x, __shfl_xor_sync(0xffffffffu, odd ? x : y, 1));
-    a = __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 2));
-    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 4));
-}
 
 // e^N = m/|m| of the mean relative velocity m (times 8), given by its component
 // in each lane; false if m = 0
@@ -212,7 +167,7 @@ __global__ void __launch_bounds__(PL_T, 4) k_particles(const ParticleArgs A, con
     const int ik = kc * cap + i;
 
     // ---- state of the particle, written before the previous lattice pass
-    const double rk = __ldcg(A.r + ik), Vk = __ldcg(A.v + ik);
+    const double rk = __ldcg(A.r_in + ik), Vk = __ldcg(A.v_in + ik);
     double fek;
     if (A.fext_in) {
         fek = A.fext_in[3 * (size_t)i + kc];
@@ -408,12 +363,12 @@ __global__ void __launch_bounds__(PL_T, 4) k_particles(const ParticleArgs A, con
         }
     }
     if (owner) {
-        A.fh[ik] = Fk;
-        A.fr[ik] = Rk;
-        if (!pin) {
-            A.v[ik] = Vn;
-            A.r[ik] = rn;
+        if (A.fh) {
+            A.fh[ik] = Fk;
+            A.fr[ik] = Rk;
         }
+        A.v[ik] = Vn;
+        A.r[ik] = rn;
         if (A.r_out) A.r_out[3 * (size_t)i + kc] = rn;
         if (A.v_out) A.v_out[3 * (size_t)i + kc] = Vn;
         if (A.done_flag) __threadfence_system();  // the host copies before the block's ticket
@@ -506,10 +461,13 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
     A.prep = s.prep;
     A.P = s.P;
     A.N = s.N;
-    A.r = s.r;
-    A.v = s.v;
-    A.fh = s.fh;
-    A.fr = s.fr;
+    const bool replay = io && io->state_out;
+    A.r_in = replay ? io->state_in : s.r;
+    A.v_in = replay ? io->state_in + 3 * (size_t)s.cap : s.v;
+    A.r = replay ? io->state_out : s.r;
+    A.v = replay ? io->state_out + 3 * (size_t)s.cap : s.v;
+    A.fh = replay ? nullptr : s.fh;
+    A.fr = replay ? nullptr : s.fr;
     A.fext = s.fext;
     A.inv_mass = s.inv_mass;
     A.gamma = s.gamma;

@@ -58,3 +58,33 @@ def test_chained_modes_and_correlator_blocks(mode):
     want = run(*args, [1] * 150, None, chain=False, lag=30)
     got = run(*args, [150], None, lag=30)
     assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("boxes,counts", [
+    ([(100, 60, 36)], [200]),           # more row segments than resident blocks: marks
+    ([(32, 16, 16)], [17]),             # a partial second block of particles, no marks
+    ([(64, 40, 40), (130, 9, 8)], [30, 0])])
+@pytest.mark.parametrize("precision", [lbp.LBP_F32, lbp.LBP_F16])
+def test_chained_adjoint_equals_plain_launches(boxes, counts, precision):
+    """Replay and reverse sweep as a chain against ordinary launches, bit for bit (no record overflows)."""
+    out = []
+    for chain in (True, False):
+        h = lbp.lbp_create_batch([(*b, 0.8) for b in boxes], precision=precision)
+        lbp.lbp_set_use_graphs(h, chain)
+        n, steps = sum(counts), 23
+        for k, ((nx, ny, nz), m) in enumerate(zip(boxes, counts)):
+            if m:
+                ps = wl.uniform_particles(m, (nz, ny, nx), 10.0, 0.5, 0.26, 1e-3, 5 + k, 6 + k)
+                lbp.lbp_particles_add_to(h, k, ps.r, ps.V * 30, ps.M, ps.gamma, ps.R)
+        lbp.lbp_particles_set_params(h, kT=1e-3, seed=3)
+        v, r = np.empty((steps, n, 3)), np.empty((steps, n, 3))
+        lbp.lbp_adjoint_record(h, steps, 9, v, r)
+        g = np.random.default_rng(1)
+        grads = {"tau": np.empty(len(boxes)), "kT": np.empty(1), "gamma": np.empty(n), "radius": np.empty(n),
+                 "mass": np.empty(n), "v0": np.empty((n, 3)), "r0": np.empty((n, 3)), "f0": np.empty((15, h.N))}
+        lbp.lbp_adjoint_backward(h, steps, g.standard_normal((steps, n, 3)), None, grads)
+        lbp.lbp_check(h)
+        lbp.lbp_destroy(h)
+        out.append([v, r, *grads.values()])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+    assert np.abs(out[0][-1]).max() > 0
