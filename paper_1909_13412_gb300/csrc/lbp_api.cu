@@ -72,6 +72,12 @@ lbp_status fail(lbp_status st, const char *fmt, ...) {
         }                                                                                \
     } while (0)
 
+#define TRY(x)                              \
+    do {                                    \
+        lbp_status st_ = (x);               \
+        if (st_ != LBP_OK) return st_;      \
+    } while (0)
+
 #define CHECK_SIM(s)                                                   \
     do {                                                               \
         if (!(s)) return fail(LBP_EINVAL, "null lbp_sim handle");      \
@@ -91,6 +97,27 @@ lbp_status leave(lbp_sim *s) {
     return LBP_OK;
 }
 
+void free_work(lbp_sim *s) {
+    if (s->work_mem) cudaFree(s->work_mem);
+    s->work_mem = nullptr;
+    s->work_bytes = 0;
+}
+
+// device memory for the handle, for which it gives up the reverse sweep's block if need be
+lbp_status handle_alloc(lbp_sim *s, void **mem, size_t bytes) {
+    cudaError_t e = cudaMalloc(mem, bytes);
+    if (e == cudaErrorMemoryAllocation && s->work_mem) {
+        (void)cudaGetLastError();
+        free_work(s);
+        e = cudaMalloc(mem, bytes);
+    }
+    if (e == cudaSuccess) return LBP_OK;
+    *mem = nullptr;
+    (void)cudaGetLastError();
+    return fail(e == cudaErrorMemoryAllocation ? LBP_ENOMEM : LBP_ECUDA, "cudaMalloc of %zu bytes: %s", bytes,
+                cudaGetErrorString(e));
+}
+
 lbp_status stage(lbp_sim *s, size_t bytes) {
     if (s->stage_bytes >= bytes) return LBP_OK;
     if (s->stage) {
@@ -99,7 +126,7 @@ lbp_status stage(lbp_sim *s, size_t bytes) {
         s->stage = nullptr;
         s->stage_bytes = 0;
     }
-    CK(cudaMalloc(&s->stage, bytes));
+    TRY(handle_alloc(s, (void **)&s->stage, bytes));
     s->stage_bytes = bytes;
     return LBP_OK;
 }
@@ -111,12 +138,6 @@ lbp_status dalloc(T **p, size_t count) {
     CK(cudaMalloc((void **)p, sizeof(T) * count));
     return LBP_OK;
 }
-
-#define TRY(x)                              \
-    do {                                    \
-        lbp_status st_ = (x);               \
-        if (st_ != LBP_OK) return st_;      \
-    } while (0)
 
 bool radius_ok(double R, int exclude) {
     if (!(R > 0.0) || !std::isfinite(R)) return false;
@@ -332,11 +353,31 @@ bool device_memory(const void *p) {
 }
 
 
-void free_tape(lbp_sim *s) {
-    if (s->tape.ck_f) cudaFree(s->tape.ck_f);
-    if (s->tape.ck_p) cudaFree(s->tape.ck_p);
-    s->tape = lbp::Tape();
+// The recording's and the reverse sweep's device memory, one block each, kept by
+// the handle: at 256^3 with 10 steps a segment, mapping and unmapping 13 GB took 9
+// of a 35 ms gradient.  A block is reused while it is large enough and not more
+// than twice what is asked; the sweep's is given back at the end of the call when
+// the two would hold more than an eighth of the device's memory, before other
+// large allocations of the handle, and when one of these fails.
+lbp_status adjoint_memory(lbp_sim *s, void **mem, size_t *have, size_t bytes) {
+    if (*mem && *have >= bytes && *have / 2 <= bytes) return LBP_OK;
+    if (*mem) cudaFree(*mem);
+    *mem = nullptr;
+    *have = 0;
+    TRY(handle_alloc(s, mem, bytes));
+    *have = bytes;
+    return LBP_OK;
 }
+
+// Split one block into arrays that start on 256-byte boundaries.
+struct Carve {
+    size_t bytes = 0;
+    size_t add(size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 255) / 256 * 256;
+        return at;
+    }
+};
 
 lbp_status host_to_device(lbp_sim *s, void *dst, const void *src, size_t bytes, int on_device) {
     CK(cudaMemcpyAsync(dst, src, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -486,12 +527,12 @@ lbp_status lbp_destroy(lbp_sim *s) {
     if (!s) return LBP_OK;
     if (s->s0) cudaStreamSynchronize(s->s0);
     if (s->s1) cudaStreamSynchronize(s->s1);
-    free_tape(s);
     void *bufs[] = {s->f[0], s->f[1], s->d_step, s->d_err, s->r, s->v, s->fh, s->fr, s->fext, s->xbuf,
                     s->mass, s->inv_mass, s->gamma, s->radius, s->sig, s->pinned, s->prep, s->fq, s->rec[0],
                     s->rec[1], s->marks[0], s->marks[1], s->ring,
                     s->d_vacf, s->vacf_sum, s->vacf_cnt, s->vacf_part, s->stage, s->inj, s->budget_part,
-                    s->corr_g, s->corr_h, s->corr_w, s->msd_state, s->msd_sum, s->ring16, s->d_xticket};
+                    s->corr_g, s->corr_h, s->corr_w, s->msd_state, s->msd_sum, s->ring16, s->d_xticket,
+                    s->tape_mem, s->work_mem};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (s->h_xflag) cudaFreeHost(s->h_xflag);
@@ -649,6 +690,7 @@ lbp_status lbp_particles_add_to(lbp_sim *s, int replica, int n, const double *r,
     if (np_new > s->cap) {
         int cap = s->cap ? s->cap : 64;
         while (cap < np_new) cap *= 2;
+        free_work(s);
         CK(cudaStreamSynchronize(s->s0));
         CK(cudaStreamSynchronize(s->s1));
         double **vec[] = {&s->r, &s->v, &s->fh, &s->fr, &s->fext};
@@ -1008,6 +1050,7 @@ lbp_status lbp_vacf_configure_ex(lbp_sim *s, int max_lag, int per_particle) {
         }
     if (max_lag < 0) return leave(s);
     if (s->np == 0) return fail(LBP_ESTATE, "lbp_vacf_configure: add particles first");
+    free_work(s);
     const int B = vacf_block_samples();
     const long long ncomp = 3ll * s->np;
     // per particle: FP32 ring of max_lag + 2 blocks (one block more than the
@@ -1234,13 +1277,16 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     if (s->np < 1) return fail(LBP_ESTATE, "lbp_adjoint_record: add particles first (the recorded outputs are their trajectories)");
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
-    free_tape(s);
+    s->tape = lbp::Tape();  // a new recording replaces the previous one
     lbp::Tape &tp = s->tape;
     const size_t pop_bytes = (size_t)storage_bytes(s->precision) * Q * s->P;
     const int64_t nck = (nsteps + checkpoint_every - 1) / checkpoint_every;
     const size_t pcount = (size_t)6 * (s->cap > 0 ? s->cap : 1);
-    TRY(dalloc(&tp.ck_f, pop_bytes * (size_t)nck));
-    TRY(dalloc(&tp.ck_p, pcount * (size_t)nck));
+    Carve c;
+    const size_t at_f = c.add(pop_bytes * (size_t)nck), at_p = c.add(sizeof(double) * pcount * (size_t)nck);
+    TRY(adjoint_memory(s, &s->tape_mem, &s->tape_bytes, c.bytes));
+    tp.ck_f = static_cast<char *>(s->tape_mem) + at_f;
+    tp.ck_p = reinterpret_cast<double *>(static_cast<char *>(s->tape_mem) + at_p);
     const size_t traj = (size_t)nsteps * s->np * 3;
     double *vt = v_traj, *rt = r_traj;
     if (!on_device && (v_traj || r_traj) && traj > 0) {
@@ -1253,11 +1299,11 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     tp.C = checkpoint_every;
     tp.np = s->np;
     tp.nck = nck;
-    Chain c{nsteps};
+    Chain chain{nsteps};
     for (int64_t n = 0; n < nsteps; ++n) {
         if (n % checkpoint_every == 0) {
             const int64_t k = n / checkpoint_every;
-            c.follows = false;  // copies follow the last step
+            chain.follows = false;  // copies follow the last step
             CK(cudaMemcpyAsync(tp.ck_f + (size_t)k * pop_bytes, s->f[s->cur], pop_bytes,
                                cudaMemcpyDeviceToDevice, s->s0));
             if (s->np > 0) {
@@ -1270,7 +1316,7 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
         // the particle kernel writes the trajectories itself
         const ParticleIO io{nullptr, rt ? rt + (size_t)n * s->np * 3 : nullptr, vt ? vt + (size_t)n * s->np * 3 : nullptr,
                             false};
-        TRY(step_once(s, c, &io));
+        TRY(step_once(s, chain, &io));
     }
     if (!on_device && traj > 0) {
         if (v_traj) CK(cudaMemcpyAsync(v_traj, vt, sizeof(double) * traj, cudaMemcpyDeviceToHost, s->s0));
@@ -1301,37 +1347,31 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
     const int nblk = adj_lattice_blocks(*s);
     const size_t rec_bytes = sizeof(unsigned long long) * REC_WORDS * (size_t)s->nseg;
 
-    // work buffers, freed on every exit path
-    char *seg = nullptr;
-    float *lam = nullptr;
-    double *dwork = nullptr;
-    struct Guard {
-        std::vector<void *> p;
-        ~Guard() {
-            for (void *q : p)
-                if (q) cudaFree(q);
-        }
-    } guard;
     // the states of a segment after its first (the first is the checkpoint itself)
-    TRY(dalloc(&seg, pop_bytes * (size_t)(C > 1 ? C - 1 : 1)));
-    guard.p.push_back(seg);
-    TRY(dalloc(&lam, (size_t)2 * Q * s->P));
-    guard.p.push_back(lam);
-    // doubles: seg_p [C][6 cap] | lam_v, lam_r [3 cap] | acc [4 np] | acc_om [nblk] |
-    //          g_v, g_r staged [traj] each
-    const size_t n_segp = (size_t)C * pcount, n_lvr = (size_t)6 * cap, n_acc = (size_t)4 * (np > 0 ? np : 1),
-                 n_om = (size_t)nblk;
+    const size_t m_max = (size_t)(C < T ? C : T);
     const bool stage_g = !on_device && traj > 0;
-    const size_t n_g = stage_g ? 2 * traj : 0;
-    TRY(dalloc(&dwork, n_segp + n_lvr + n_acc + n_om + n_g));
-    guard.p.push_back(dwork);
-    double *f0tmp = nullptr;  // FP64 staging of dL/df0 for a host destination
-    if (out->f0 && !on_device) {
-        TRY(dalloc(&f0tmp, (size_t)Q * s->N));
-        guard.p.push_back(f0tmp);
-    }
-    double *seg_p = dwork, *lam_v = seg_p + n_segp, *lam_r = lam_v + 3 * (size_t)cap,
-           *acc = lam_v + n_lvr, *acc_om = acc + n_acc, *gst = acc_om + n_om;
+    const size_t n_lvr = (size_t)6 * cap, n_acc = (size_t)4 * (np > 0 ? np : 1), n_om = (size_t)nblk;
+    Carve c;
+    const size_t at_seg = c.add(pop_bytes * (m_max - 1)), at_lam = c.add(sizeof(float) * 2 * Q * s->P),
+                 at_segp = c.add(sizeof(double) * m_max * pcount),  // particle states, likewise
+                 at_lvr = c.add(sizeof(double) * (n_lvr + n_acc + n_om)),
+                 at_g = c.add(stage_g ? sizeof(double) * 2 * traj : 0),
+                 at_f0 = c.add(out->f0 && !on_device ? sizeof(double) * Q * s->N : 0);  // dL/df0 for a host destination
+    TRY(adjoint_memory(s, &s->work_mem, &s->work_bytes, c.bytes));
+    // given back at the end if it is much
+    struct Guard {
+        lbp_sim *s;
+        ~Guard() {
+            size_t free_b = 0, total = 0;
+            if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || s->tape_bytes + s->work_bytes > total / 8) free_work(s);
+        }
+    } guard{s};
+    char *work = static_cast<char *>(s->work_mem);
+    char *seg = work + at_seg;
+    float *lam = reinterpret_cast<float *>(work + at_lam);
+    double *seg_p = reinterpret_cast<double *>(work + at_segp), *lam_v = reinterpret_cast<double *>(work + at_lvr),
+           *lam_r = lam_v + 3 * (size_t)cap, *acc = lam_v + n_lvr, *acc_om = acc + n_acc,
+           *gst = reinterpret_cast<double *>(work + at_g), *f0tmp = reinterpret_cast<double *>(work + at_f0);
     const double *gv = g_v, *gr = g_r;
     if (stage_g) {
         if (g_v) {
@@ -1343,7 +1383,7 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
             gr = gst + traj;
         }
     }
-    CK(cudaMemsetAsync(lam, 0, sizeof(float) * 2 * Q * s->P, s->s0));
+    CK(cudaMemsetAsync(lam, 0, sizeof(float) * Q * s->P, s->s0));  // the other one is written first
     CK(cudaMemsetAsync(lam_v, 0, sizeof(double) * (n_lvr + n_acc + n_om), s->s0));
     const int saved_vacf = s->vacf_lag;
     s->vacf_lag = -1;  // the replay writes no VACF samples
@@ -1443,7 +1483,7 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
                 CK(cudaMemcpyAsync(out->f0, f0tmp, sizeof(double) * Q * s->N, cudaMemcpyDeviceToHost, s->s0));
         }
         if (np > 0) {
-            double *aos = seg_p;  // free now: C * 6 cap >= 6 np doubles
+            double *aos = seg_p;  // free now: at least 6 cap doubles
             if (out->v0) {
                 CK(launch_soa_to_aos(lam_v, on_device ? out->v0 : aos, np, cap, s->s0));
                 if (!on_device)

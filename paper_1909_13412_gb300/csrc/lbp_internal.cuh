@@ -526,6 +526,10 @@ struct Sim {
     double *msd_sum = nullptr;    // [K + 1]
 
     Tape tape;
+    // device memory of the recording and of the reverse sweep, kept for the next
+    // ones (see adjoint_memory in lbp_api.cu)
+    void *tape_mem = nullptr, *work_mem = nullptr;
+    size_t tape_bytes = 0, work_bytes = 0;
     uint64_t edits = 0;  // state-changing calls other than steps (set_*, add)
 
     // conservation budget: momentum put into the unpinned particles by F_R and
