@@ -357,14 +357,17 @@ __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__
                                                      long long P, const RepTable<MAXR> rt,
                                                      const unsigned long long *rec_cur,
                                                      unsigned long long *rec_prev, double *fqd,
-                                                     long long N, double *acc_omega, const Marks mk) {
+                                                     long long N, double *acc_omega, const Marks mk, bool flip) {
     __shared__ float s_red[SEG / 32];
-    // the block's box (batches: one block per row segment of every box, in box order)
-    const int rb = find_block_rep(rt, blockIdx.x);
+    // the block's box (batches: one block per row segment of every box, in box
+    // order); consecutive reverse steps run through them in opposite directions,
+    // so that each first reads what the one before wrote last (in L2)
+    const unsigned block = flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int rb = find_block_rep(rt, block);
     const Rep &rp = rt.rep[rb];
     const int nx = rp.nx, ny = rp.ny, nz = rp.nz, nchunks = rp.nchunks;
     const float omega = rp.omega;
-    const unsigned item = blockIdx.x - rt.item_off[rb];
+    const unsigned item = block - rt.item_off[rb];
     const unsigned row = divide(item, rp.dchunks);
     const int chunk = (int)(item - row * (unsigned)nchunks);
     const size_t seg = (size_t)rp.seg_off + (size_t)row * nchunks + chunk;
@@ -478,7 +481,7 @@ __global__ void __launch_bounds__(SEG, 6) k_adj_lattice(const typename St::T *__
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < SEG / 32; ++w) s += s_red[w];
-        acc_omega[blockIdx.x] = __ldcg(acc_omega + blockIdx.x) + (double)s;
+        acc_omega[block] = __ldcg(acc_omega + block) + (double)s;
     }
 }
 
@@ -570,7 +573,7 @@ cudaError_t launch_adj_lattice(Sim &s, const AdjStep &a, cudaStream_t st, bool p
             const unsigned long long *rec = s.rec[a.parity];
             return launch_k(k_adj_lattice<St, MAXR>, grid, SEG, 0, st, pdl, static_cast<const typename St::T *>(a.g),
                             a.lam, a.lam_out, (long long)s.P, rt, rec, s.rec[a.parity ^ 1],
-                            reinterpret_cast<double *>(s.fq), (long long)s.N, a.acc_omega, mk);
+                            reinterpret_cast<double *>(s.fq), (long long)s.N, a.acc_omega, mk, a.parity != 0);
         });
     });
 }

@@ -167,7 +167,7 @@ lbp_status enqueue_step(lbp_sim *s, bool timed, bool chained, unsigned epoch, un
     if (s->np > 0)
         CK(launch_stream_collide_forced(*s, src, dst, parity, s->s0, !timed, epoch));
     else
-        CK(launch_stream_collide(*s, src, dst, s->s0));
+        CK(launch_stream_collide(*s, src, dst, parity, s->s0, chained));
     if (timed) {
         CK(cudaEventRecord(s->tev[2 * s->ntimed + 1], s->s0));
         s->ntimed += 1;
@@ -479,6 +479,7 @@ lbp_status lbp_create_batch(const lbp_lattice_desc *descs, int nrep, void *strea
     };
     cudaError_t e = cudaGetDevice(&s->dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->l2_bytes, cudaDevAttrL2CacheSize, s->dev);
     if (e == cudaSuccess) e = prepare_lbm_kernels();
     if (e == cudaSuccess) e = prepare_vacf_kernels();
     // the step's own kernels at the highest stream priority, the side stream (the

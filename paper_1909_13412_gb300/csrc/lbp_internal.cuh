@@ -47,6 +47,32 @@ __host__ __device__ constexpr float wgtf(int a) {
 //          |g/w| up to 64 still fits.
 constexpr float F16_SCALE = 1024.f;
 
+// A population load of a lattice pass that is the line's last use before the line
+// is overwritten (two steps on): through L2, first to be evicted.
+__device__ __forceinline__ unsigned long long evict_first() {
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ float load_last(const float *a) {
+    float v;
+    asm("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(evict_first()) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned short load_last(const unsigned short *a) {
+    unsigned short v;
+    asm("ld.global.cg.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(evict_first()) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 load_last(const uint2 *a) {
+    uint2 v;
+    asm("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+        : "=r"(v.x), "=r"(v.y)
+        : "l"(a), "l"(evict_first())
+        : "memory");
+    return v;
+}
+
 // load/store: the deviation g (gather: the same load through L2).  cload/cstore (and cload_shared): the values
 // the lattice kernels' collision works on (collide_st): g itself for F32 and
 // BF16; for F16 the stored variable h = g F16_SCALE / w_a, on which the
@@ -60,7 +86,11 @@ struct StoreF32 {
     static __device__ __forceinline__ float load_shared(const T *p, int) { return *p; }
     static __device__ __forceinline__ void store(T *p, int, float v) { *p = v; }
     // through L2: a chained step reads populations before its launch dependency resolves
-    static __device__ __forceinline__ float cload(const T *p, int) { return __ldcg(p); }
+    template <bool LAST>
+    static __device__ __forceinline__ float cload(const T *p, int) {
+        if constexpr (LAST) return load_last(p);
+        return __ldcg(p);
+    }
     static __device__ __forceinline__ float cload_shared(const T *p, int a) { return load_shared(p, a); }
     static __device__ __forceinline__ void cstore(T *p, int a, float v) { store(p, a, v); }
 };
@@ -71,7 +101,11 @@ struct StoreBF16 {
     static __device__ __forceinline__ float gather(const T *p, int) { return __bfloat162float(__ldcg(p)); }
     static __device__ __forceinline__ float load_shared(const T *p, int) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store(T *p, int, float v) { *p = __float2bfloat16_rn(v); }
-    static __device__ __forceinline__ float cload(const T *p, int) { return __bfloat162float(__ldcg(p)); }
+    template <bool LAST>
+    static __device__ __forceinline__ float cload(const T *p, int) {
+        if constexpr (LAST) return __uint_as_float((unsigned)load_last(reinterpret_cast<const unsigned short *>(p)) << 16);
+        return __bfloat162float(__ldcg(p));
+    }
     static __device__ __forceinline__ float cload_shared(const T *p, int a) { return load_shared(p, a); }
     static __device__ __forceinline__ void cstore(T *p, int a, float v) { store(p, a, v); }
 };
@@ -90,7 +124,11 @@ struct StoreF16 {
     static __device__ __forceinline__ void store(T *p, int a, float v) {
         *p = __float2half_rn(v * (F16_SCALE / wgtf(a)));
     }
-    static __device__ __forceinline__ float cload(const T *p, int) { return __half2float(__ldcg(p)); }
+    template <bool LAST>
+    static __device__ __forceinline__ float cload(const T *p, int) {
+        if constexpr (LAST) return __half2float(__ushort_as_half(load_last(reinterpret_cast<const unsigned short *>(p))));
+        return __half2float(__ldcg(p));
+    }
     static __device__ __forceinline__ float cload_shared(const T *p, int) { return __half2float(*p); }
     static __device__ __forceinline__ void cstore(T *p, int, float v) { *p = __float2half_rn(v); }
 };
@@ -467,6 +505,7 @@ struct Sim {
     int variant = 0;  // lattice kernel: 0 one node per thread, 1 two nodes, 2 bulk-copy staged
     int dev = 0;
     int num_sms = 0;
+    int l2_bytes = 0;
     long long wait_cycles = DEFAULT_WAIT_CYCLES;  // bound of every device-side wait (SM cycles)
     int wait_probe = 0;  // 1: the staged kernel's waits run out on purpose (tests of the error path)
 
@@ -583,7 +622,9 @@ cudaError_t launch_k(void (*kern)(KArgs...), unsigned grid, unsigned block, size
 // ------------------------------------------------------------ launchers
 // lbm_kernels.cu
 cudaError_t prepare_lbm_kernels();
-cudaError_t launch_stream_collide(Sim &s, const void *src, void *dst, cudaStream_t st);
+// parity: of the step (its direction where passes alternate); chained: right after the pass of the step before
+cudaError_t launch_stream_collide(Sim &s, const void *src, void *dst, int parity, cudaStream_t st,
+                                  bool chained = false);
 // the lattice kernels with an explicit step counter, force records and rows per block
 cudaError_t launch_stream_collide_cfg(Sim &s, const void *src, void *dst, long long *bump,
                                       int rows, int variant, cudaStream_t st);
@@ -594,6 +635,7 @@ cudaError_t launch_stream_collide_forced_cfg(Sim &s, const void *src, void *dst,
 void default_shape(const Sim &s, int &rows, int &variant);  // before lbp_autotune
 bool pair_kernel_ok(const Sim &s);  // 2-byte storage and every box with even nx
 bool variant_ok(const Sim &s, int variant);
+bool sweeps_back(const Sim &s);  // consecutive passes run in opposite order (see lbm_kernels.cu)
 bool lattice_chains(const Sim &s);  // the handle's lattice kernel reads ahead through L2
 bool lattice_marks(const Sim &s);   // ... and gains from marks (Marks)
 // pdl: launched right after the step's particle kernel on `st`, as its

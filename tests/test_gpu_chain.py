@@ -39,6 +39,7 @@ def run(boxes, counts, precision, mode, calls, shape, chain=True, lag=-1):
     ([(32, 32, 32)], [1]),              # a few marked rows
     ([(3, 5, 131)], [40]),              # corners that wrap in every direction, records that overflow
     ([(260, 9, 8)], [300]),             # three segments a row, most rows marked
+    ([(128, 80, 72)], [500]),           # more row segments than resident warps of the four-node kernel
     ([(96, 64, 64)], [9000]),           # enough particles for the other order of preparation
     ([(64, 64, 64)], [20000]),          # more particle blocks than are resident at a time
     ([(64, 20, 20), (17, 9, 30), (130, 8, 8)], [2, 0, 30])])
