@@ -40,6 +40,7 @@ def run(boxes, counts, precision, mode, calls, shape, chain=True, lag=-1):
     ([(3, 5, 131)], [40]),              # corners that wrap in every direction, records that overflow
     ([(260, 9, 8)], [300]),             # three segments a row, most rows marked
     ([(128, 80, 72)], [500]),           # more row segments than resident warps of the four-node kernel
+    ([(33, 21, 19), (32, 7, 9), (5, 4, 3)], [9, 3, 1]),  # short rows
     ([(96, 64, 64)], [9000]),           # enough particles for the other order of preparation
     ([(64, 64, 64)], [20000]),          # more particle blocks than are resident at a time
     ([(64, 20, 20), (17, 9, 30), (130, 8, 8)], [2, 0, 30])])
@@ -64,6 +65,7 @@ def test_chained_modes_and_correlator_blocks(mode):
 @pytest.mark.parametrize("boxes,counts", [
     ([(100, 60, 36)], [200]),           # more row segments than resident blocks: marks
     ([(32, 16, 16)], [17]),             # a partial second block of particles, no marks
+    ([(64, 63, 61)], [40]),             # an odd number of rows
     ([(64, 40, 40), (130, 9, 8)], [30, 0])])
 @pytest.mark.parametrize("precision", [lbp.LBP_F32, lbp.LBP_F16])
 def test_chained_adjoint_equals_plain_launches(boxes, counts, precision):
