@@ -336,17 +336,17 @@ __global__ void __launch_bounds__(PAIR_BX) k_stream_collide_pair(
         for (int a = 0; a < Q; ++a) {
             const int rb = drow[h] + n.oy[ey(a) + 1] + n.oz[ez(a) + 1];  // source row start
             const unsigned *src = reinterpret_cast<const unsigned *>(pl.s[a] + rb);
-            const unsigned v = __ldg(src + (x >> 1));
+            const unsigned v = __ldcg(src + (x >> 1));  // ahead of the wait: through L2
             unsigned w = v;
             if (ex(a) > 0) {
                 // pull from x - 1: (x - 1, x) = (hi of left pair, lo of own)
                 unsigned left = __shfl_up_sync(0xffffffffu, v, 1);
-                if (own_left) left = __ldg(src + (xl >> 1));
+                if (own_left) left = __ldcg(src + (xl >> 1));
                 w = __byte_perm(left, v, 0x5432);
             } else if (ex(a) < 0) {
                 // pull from x + 1: (x + 1, x + 2) = (hi of own, lo of right pair)
                 unsigned right = __shfl_down_sync(0xffffffffu, v, 1);
-                if (own_right) right = __ldg(src + (xr >> 1));
+                if (own_right) right = __ldcg(src + (xr >> 1));
                 w = __byte_perm(v, right, 0x5432);
             }
             unpack2<St>(w, a, g[h][0][a], g[h][1][a]);

@@ -45,9 +45,11 @@ def run(boxes, counts, precision, mode, calls, shape, chain=True, lag=-1):
     ([(64, 64, 64)], [20000]),          # more particle blocks than are resident at a time
     ([(64, 20, 20), (17, 9, 30), (130, 8, 8)], [2, 0, 30])])
 @pytest.mark.parametrize("precision,shape", [
-    (lbp.LBP_F32, None), (lbp.LBP_F32, (1, 0)), (lbp.LBP_F32, (4, 0)), (lbp.LBP_BF16, (2, 0)), (lbp.LBP_F16, None),
+    (lbp.LBP_F32, None), (lbp.LBP_F32, (1, 0)), (lbp.LBP_F32, (4, 0)), (lbp.LBP_BF16, (2, 0)), (lbp.LBP_F16, None), (lbp.LBP_F16, (2, 1)),
     (lbp.LBP_BF16, None)])
 def test_steps_of_one_call_equal_single_calls(boxes, counts, precision, shape):
+    if shape == (2, 1) and any(b[0] % 2 for b in boxes):
+        pytest.skip("two nodes per thread need even rows")
     want = run(boxes, counts, precision, lbp.LBP_STOKESLET, [1] * 40, shape, chain=False)
     for calls in ([40], [7, 33]):
         got = run(boxes, counts, precision, lbp.LBP_STOKESLET, calls, shape)
