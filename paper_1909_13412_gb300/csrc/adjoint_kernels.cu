@@ -219,16 +219,18 @@ __global__ void __launch_bounds__(AP_T, 3) k_adj_particles(const AdjPArgs A, con
         }
     }
     const double F[3] = {from_comp(FH, 0), from_comp(FH, 1), from_comp(FH, 2)};
+    int next_seg = 0;  // the row segment of corner p of the next reverse step's cell
     if (A.marks && A.prev_r) {
-        // mark the row segment of corner p of the next reverse step's cell
         const int b = (int)floor(__ldcg(A.prev_r + ik));
         const int x1 = wrapi(from_comp(b, 0) + c0, nx), y1 = wrapi(from_comp(b, 1) + c1, ny),
                   z1 = wrapi(from_comp(b, 2) + c2, nz);
-        if (live) A.marks[rp.seg_off + ((long long)z1 * ny + y1) * rp.nchunks + x1 / SEG] = A.mark_epoch;
+        next_seg = (int)(rp.seg_off + ((long long)z1 * ny + y1) * rp.nchunks + x1 / SEG);
     }
 
     // ---- the lattice kernel of the reverse step before is complete
+    // (it read its marks from the array that the next step's go to)
     grid_dependency_wait();
+    if (A.marks && A.prev_r && live) A.marks[next_seg] = A.mark_epoch;
     double lq = 0.0, lu[3] = {0.0, 0.0, 0.0};  // adjoints of q (component kc) and of u(x_p)
     if (A.mode != LBP_BROWNIAN) {
         // lam_F(x_p) (aligned): dL/dfhat_a(x_p) = dL/df^{n+1}_a(x_p + e_a), the buffer's layout

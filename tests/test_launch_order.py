@@ -1,0 +1,56 @@
+"""What the chained kernels may do before their launch dependency resolves, read from their source.
+
+A kernel of the chain may start before the kernel ahead of it has finished, so
+what it writes or reads ahead of grid_dependency_wait is part of its
+correctness, and a run shows a mistake there only when the timing is unlucky.
+"""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1909_13412_gb300", "csrc")
+
+
+def source(name):
+    """The file without its comments."""
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def block(text, at):
+    """The braced block that opens at or after position `at`."""
+    i = text.index("{", at)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return text[i:j + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def kernel(name, file):
+    text = source(file)
+    m = re.search(r"__global__[^;{]*?\b" + name + r"\(", text)
+    # past the parameter list
+    return block(text, text.index(")", text.index(name + "(", m.start())))
+
+
+@pytest.mark.parametrize("name,file,allowed", [
+    # the external forces of an exchange step, whose particle kernel is never chained
+    ("k_particles", "particle_kernels.cu", {"fext"}),
+    ("k_adj_particles", "adjoint_kernels.cu", set())])
+def test_particle_kernels_write_nothing_ahead_of_their_dependency(name, file, allowed):
+    """The lattice kernel before may still be running: it reads the marks, the
+    records and the accumulators that these kernels write."""
+    body = kernel(name, file)
+    parts = body.split("grid_dependency_wait();")
+    assert len(parts) == 3  # the triggering warp's, and the others'
+    ahead = parts[0] + parts[1]
+    written = re.findall(r"\bA\.(\w+)\s*\[[^;=]*\]\s*[-+|]?=[^=]", ahead)
+    written += re.findall(r"\*\s*A\.(\w+)\s*[-+|]?=[^=]", ahead)
+    written += re.findall(r"atomic\w+\(\s*A\.(\w+)", ahead)
+    assert set(written) <= allowed
+    # and the same search finds the stores that come after
+    after = re.findall(r"\bA\.(\w+)\s*\[[^;=]*\]\s*[-+|]?=[^=]", parts[2])
+    assert "marks" in after
