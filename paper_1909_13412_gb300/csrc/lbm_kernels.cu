@@ -451,11 +451,6 @@ constexpr int QUAD_WARPS = 2;  // row segments (warps) per block
 // cached, unmarked kernel was at 213.0 / 215.3.  More rows keep more loads in
 // flight and need the registers.
 
-template <typename St>
-__device__ __forceinline__ unsigned short load_elem(const typename St::T *p) {
-    return __ldcg(reinterpret_cast<const unsigned short *>(p));
-}
-
 template <typename St, int R, int MAXR, bool FORCED, bool BACK>
 __global__ void __launch_bounds__(32 * QUAD_WARPS, R == 1 ? 14 : 1) k_stream_collide_quad(
     Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *rec_cur,
@@ -500,8 +495,8 @@ __global__ void __launch_bounds__(32 * QUAD_WARPS, R == 1 ? 14 : 1) k_stream_col
             const uint2 *at = reinterpret_cast<const uint2 *>(src + x);
             p[h][a] = BACK ? load_last(at) : __ldcg(at);
             edge[h][a] = 0;
-            if (ex(a) > 0 && own_left) edge[h][a] = load_elem<St>(src + xl);
-            if (ex(a) < 0 && own_right) edge[h][a] = load_elem<St>(src + xr);
+            if (ex(a) > 0 && own_left) edge[h][a] = load_word(src + xl);
+            if (ex(a) < 0 && own_right) edge[h][a] = load_word(src + xr);
         }
     }
     if (FORCED) {

@@ -56,21 +56,28 @@ __device__ __forceinline__ unsigned long long evict_first() {
 }
 __device__ __forceinline__ float load_last(const float *a) {
     float v;
-    asm("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(evict_first()) : "memory");
+    asm volatile("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(evict_first()) : "memory");
     return v;
 }
 __device__ __forceinline__ unsigned short load_last(const unsigned short *a) {
     unsigned short v;
-    asm("ld.global.cg.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(evict_first()) : "memory");
+    asm volatile("ld.global.cg.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(evict_first()) : "memory");
     return v;
 }
 __device__ __forceinline__ uint2 load_last(const uint2 *a) {
     uint2 v;
-    asm("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+    asm volatile("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
         : "=r"(v.x), "=r"(v.y)
         : "l"(a), "l"(evict_first())
         : "memory");
     return v;
+}
+
+// A 2-byte population through L2.  Loads that must stay behind grid_dependency_wait
+// are volatile asm: the toolkit's __ldcg is for words like this one, but not for
+// __half and __nv_bfloat16, whose loads the compiler may move ahead of the wait.
+__device__ __forceinline__ unsigned short load_word(const void *p) {
+    return __ldcg(static_cast<const unsigned short *>(p));
 }
 
 // load/store: the deviation g (gather: the same load through L2).  cload/cstore (and cload_shared): the values
@@ -98,13 +105,13 @@ struct StoreBF16 {
     using T = __nv_bfloat16;
     static constexpr bool SCALED = false;
     static __device__ __forceinline__ float load(const T *p, int) { return __bfloat162float(__ldg(p)); }
-    static __device__ __forceinline__ float gather(const T *p, int) { return __bfloat162float(__ldcg(p)); }
+    static __device__ __forceinline__ float gather(const T *p, int) { return __uint_as_float((unsigned)load_word(p) << 16); }
     static __device__ __forceinline__ float load_shared(const T *p, int) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store(T *p, int, float v) { *p = __float2bfloat16_rn(v); }
     template <bool LAST>
     static __device__ __forceinline__ float cload(const T *p, int) {
         if constexpr (LAST) return __uint_as_float((unsigned)load_last(reinterpret_cast<const unsigned short *>(p)) << 16);
-        return __bfloat162float(__ldcg(p));
+        return __uint_as_float((unsigned)load_word(p) << 16);
     }
     static __device__ __forceinline__ float cload_shared(const T *p, int a) { return load_shared(p, a); }
     static __device__ __forceinline__ void cstore(T *p, int a, float v) { store(p, a, v); }
@@ -116,7 +123,7 @@ struct StoreF16 {
         return __half2float(__ldg(p)) * (wgtf(a) * (1.f / F16_SCALE));
     }
     static __device__ __forceinline__ float gather(const T *p, int a) {
-        return __half2float(__ldcg(p)) * (wgtf(a) * (1.f / F16_SCALE));
+        return __half2float(__ushort_as_half(load_word(p))) * (wgtf(a) * (1.f / F16_SCALE));
     }
     static __device__ __forceinline__ float load_shared(const T *p, int a) {
         return __half2float(*p) * (wgtf(a) * (1.f / F16_SCALE));
@@ -127,7 +134,7 @@ struct StoreF16 {
     template <bool LAST>
     static __device__ __forceinline__ float cload(const T *p, int) {
         if constexpr (LAST) return __half2float(__ushort_as_half(load_last(reinterpret_cast<const unsigned short *>(p))));
-        return __half2float(__ldcg(p));
+        return __half2float(__ushort_as_half(load_word(p)));
     }
     static __device__ __forceinline__ float cload_shared(const T *p, int) { return __half2float(*p); }
     static __device__ __forceinline__ void cstore(T *p, int, float v) { *p = __float2half_rn(v); }

@@ -54,3 +54,40 @@ def test_particle_kernels_write_nothing_ahead_of_their_dependency(name, file, al
     # and the same search finds the stores that come after
     after = re.findall(r"\bA\.(\w+)\s*\[[^;=]*\]\s*[-+|]?=[^=]", parts[2])
     assert "marks" in after
+
+
+CUDA_INCLUDE = "/usr/local/cuda/include"
+
+
+def cuda_headers():
+    found = ""
+    for f in ("sm_32_intrinsics.hpp", "cuda_fp16.hpp", "cuda_bf16.hpp"):
+        path = os.path.join(CUDA_INCLUDE, f)
+        if not os.path.exists(path):
+            pytest.skip("needs the CUDA toolkit's headers")
+        found += open(path).read()
+    return found
+
+
+def volatile_ldcg(header, ctype):
+    """Whether the toolkit's __ldcg of this type is a volatile asm: a plain one may move across the wait's."""
+    m = re.search(r"__ldcg\(\s*const\s+" + ctype + r"\s*\*[^)]*\)\s*\{(.*?)\}", header, flags=re.S)
+    return re.search(r"\basm\s+volatile\b", m.group(1)) is not None
+
+
+def test_two_byte_populations_are_loaded_as_volatile_words():
+    header = cuda_headers()
+    for ctype in ("float", "double", "int", "unsigned int", "unsigned short", "uint2", "long long", "unsigned long long"):
+        assert volatile_ldcg(header, ctype), ctype
+    if volatile_ldcg(header, "__half") and volatile_ldcg(header, "__nv_bfloat16"):
+        pytest.skip("this toolkit orders the 2-byte types' loads too")
+    text = source("lbp_internal.cuh")
+    for store in ("StoreBF16", "StoreF16"):
+        body = block(text, text.index("struct " + store))
+        assert "__ldcg(" not in body, store  # of its 2-byte type: see load_word
+        for fn in ("gather", "cload"):
+            assert re.search(r"load_(word|last)\(", block(body, body.index(" " + fn + "("))), (store, fn)
+    assert "const unsigned short *" in block(text, text.index("unsigned short load_word("))
+    # the hinted loads are asm of this library
+    for m in re.finditer(r"load_last\(const [^)]*\)", text):
+        assert "asm volatile" in block(text, m.end()), m.group(0)
