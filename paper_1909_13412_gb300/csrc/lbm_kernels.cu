@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(PAIR_BX) k_stream_collide_pair(
                     const int d = drow[h] + x;
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        s0[k] += (long long)fq[k * Ntot + d];
-                        s1[k] += (long long)fq[k * Ntot + d + 1];
+                        s0[k] += (long long)__ldcg(fq + k * Ntot + d);
+                        s1[k] += (long long)__ldcg(fq + k * Ntot + d + 1);
                         fq[k * Ntot + d] = 0ull;
                         fq[k * Ntot + d + 1] = 0ull;
                     }
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(32 * QUAD_WARPS, R == 1 ? 14 : 1) k_stream_col
                     for (int k = 0; k < 4; ++k)
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            sum[k][c] += (long long)fq[c * Ntot + d + k];
+                            sum[k][c] += (long long)__ldcg(fq + c * Ntot + d + k);
                             fq[c * Ntot + d + k] = 0ull;
                         }
                 }

@@ -211,9 +211,9 @@ __global__ void __launch_bounds__(STAGED_THREADS + 32) k_stream_collide_staged(
                             a2 += (long long)rec[REC_F0 + 3 * sl + 2];
                         }
                     if (cnt > REC_SLOTS) {
-                        a0 += (long long)fq[d];
-                        a1 += (long long)fq[Ntot + d];
-                        a2 += (long long)fq[2 * Ntot + d];
+                        a0 += (long long)__ldcg(fq + d);
+                        a1 += (long long)__ldcg(fq + Ntot + d);
+                        a2 += (long long)__ldcg(fq + 2 * Ntot + d);
                         fq[d] = 0ull;
                         fq[Ntot + d] = 0ull;
                         fq[2 * Ntot + d] = 0ull;

@@ -91,3 +91,17 @@ def test_two_byte_populations_are_loaded_as_volatile_words():
     # the hinted loads are asm of this library
     for m in re.finditer(r"load_last\(const [^)]*\)", text):
         assert "asm volatile" in block(text, m.end()), m.group(0)
+
+
+@pytest.mark.parametrize("name,file", [
+    ("k_stream_collide_forced", "lbm_kernels.cu"), ("k_stream_collide_pair", "lbm_kernels.cu"),
+    ("k_stream_collide_quad", "lbm_kernels.cu"), ("k_stream_collide_staged", "lbm_staged.cu"),
+    ("k_adj_lattice", "adjoint_kernels.cu")])
+def test_force_overflow_is_read_through_l2(name, file):
+    """The accumulators are added to by atomics of other kernels of the chain, and
+    an SM may still hold the line in L1 from a step before."""
+    body = kernel(name, file)
+    reads = re.findall(r"[^\n;]*\bfqd?\s*(?:\[|\+)[^;]*;", body)
+    reads = [r for r in reads if not re.search(r"\bfqd?\s*\[[^=]*\]\s*=[^=]", r)]
+    assert reads or "__ldcg(fq" in body
+    assert all("__ldcg(fq" in r for r in reads), reads
