@@ -597,7 +597,7 @@ int adj_lattice_first_block(const Sim &s, int replica) {
 
 // dL/dfhat_a(y) of the first recorded state = dL/df_a(y + e_a) of its first
 // step (the buffer's layout), to the FP64 [15][N] ABI layout, every box periodic on its own.
-// One block per row segment, its 15 values a thread in flight together, widened
+// A block serves SEG consecutive nodes, 15 values a thread in flight together, widened
 // on their bits: the FP64 pipe and two 64-bit divisions a value took 1.75 ms at
 // 256^3, the bytes take 0.45 ms; measured 0.44 ms.
 template <int MAXR>
@@ -606,13 +606,13 @@ __global__ void __launch_bounds__(SEG) k_adj_out(const float *__restrict__ src, 
     const int rb = find_block_rep(rt, blockIdx.x);
     const Rep &rp = rt.rep[rb];
     const int nx = rp.nx, ny = rp.ny, nz = rp.nz;
-    const unsigned item = blockIdx.x - rt.item_off[rb];
-    const unsigned row = divide(item, rp.dchunks);
-    const int x = (int)(item - row * (unsigned)rp.nchunks) * SEG + threadIdx.x;
-    if (x >= nx) return;
+    const unsigned node = (blockIdx.x - rt.item_off[rb]) * SEG + threadIdx.x;
+    if (node >= (unsigned)nx * ny * nz) return;
+    const unsigned row = divide(node, rp.dchunks);  // see node_table
+    const int x = (int)(node - row * (unsigned)nx);
     const int z = (int)divide(row, rp.dny), y = (int)(row - (unsigned)z * ny);
     const int slab = nx * ny;
-    const long long i = rp.node_off + (long long)row * nx + x;
+    const long long i = rp.node_off + node;
     // offsets of x + e (index e + 1), periodic
     const int ox[3] = {x == 0 ? nx - 1 : -1, 0, x == nx - 1 ? 1 - nx : 1};
     const int oy[3] = {y == 0 ? (ny - 1) * nx : -nx, 0, y == ny - 1 ? (1 - ny) * nx : nx};
@@ -626,11 +626,12 @@ __global__ void __launch_bounds__(SEG) k_adj_out(const float *__restrict__ src, 
 }
 
 cudaError_t launch_f32_to_f64(Sim &s, const float *src, double *dst, cudaStream_t st) {
-    return by_batch_adj(s, [&](const auto &rt) {
+    auto launch = [&](const auto &rt) {
         constexpr int MAXR = sizeof(rt.rep) / sizeof(Rep);
         k_adj_out<MAXR><<<rt.item_off[rt.nrep], SEG, 0, st>>>(src, dst, rt, s.N, s.P);
         return cudaGetLastError();
-    });
+    };
+    return s.nrep == 1 ? launch(node_table<1>(s)) : launch(node_table<MAX_BATCH>(s));
 }
 
 }  // namespace lbp

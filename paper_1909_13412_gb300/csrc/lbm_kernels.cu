@@ -994,8 +994,9 @@ cudaError_t launch_budget(Sim &s, const void *src, double *out, cudaStream_t st)
 // whose mantissa then holds the part as an integer.  A node with a value
 // that does not split exactly (below 2^(E - 18), with bits under 2^(E - 41)),
 // with a huge, an infinite or a NaN value takes the FP64 additions, as does a
-// value range near the FP32 denormals.  One block per row segment, as the
-// lattice pass.  Measured with u read: 2.28 -> 0.25 ms at 256^3 (BF16 storage),
+// value range near the FP32 denormals.  A block serves SEG consecutive nodes,
+// whatever the rows (with one block per row segment, rows of one node took 2.11 ms
+// for 4 M nodes, now 0.07).  Measured with u read: 2.28 -> 0.25 ms at 256^3 (BF16 storage),
 // 5.86 -> 0.92 ms for 68 boxes of 43 M nodes (FP32).
 // ---------------------------------------------------------------------------
 struct Moments {
@@ -1061,10 +1062,10 @@ __global__ void __launch_bounds__(SEG) k_fields(const typename St::T *__restrict
                                                 double *p, const RepTable<MAXR> rt, long long N, long long P) {
     const int r = find_block_rep(rt, blockIdx.x);
     const Rep &rp = rt.rep[r];
-    const unsigned item = blockIdx.x - rt.item_off[r];
-    const unsigned row = divide(item, rp.dchunks);
-    const int x = (int)(item - row * (unsigned)rp.nchunks) * SEG + threadIdx.x;
-    if (x >= rp.nx) return;
+    const unsigned node = (blockIdx.x - rt.item_off[r]) * SEG + threadIdx.x;
+    if (node >= (unsigned)rp.nx * rp.ny * rp.nz) return;
+    const unsigned row = divide(node, rp.dchunks);  // see node_table
+    const int x = (int)(node - row * (unsigned)rp.nx);
     const NodeIdx n = node_index(x, row, rp.nx, rp.ny, rp.nz, rp.dny);
     const long long i = rp.node_off + n.d;
     float g[Q];
@@ -1085,12 +1086,13 @@ cudaError_t launch_fields(Sim &s, const void *src, double *rho, double *u, doubl
                           cudaStream_t st) {
     return by_storage(s, [&](auto tag) {
         using St = decltype(tag);
-        return by_batch(s, 1, [&](const auto &rt) {
+        auto launch = [&](const auto &rt) {
             constexpr int MAXR = sizeof(rt.rep) / sizeof(Rep);
             k_fields<St, MAXR><<<rt.item_off[rt.nrep], SEG, 0, st>>>(static_cast<const typename St::T *>(src), rho, u,
                                                                      p, rt, s.N, s.P);
             return cudaGetLastError();
-        });
+        };
+        return s.nrep == 1 ? launch(node_table<1>(s)) : launch(node_table<MAX_BATCH>(s));
     });
 }
 

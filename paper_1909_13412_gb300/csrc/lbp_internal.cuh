@@ -608,6 +608,24 @@ struct Sim {
     int64_t timed_launches = 0;
 };
 
+// The box table of a readout whose blocks serve SEG consecutive nodes of a box each
+// (item_off counts those blocks), so that short rows fill them too; dchunks divides
+// a node by nx here.
+template <int MAXR>
+RepTable<MAXR> node_table(const Sim &s) {
+    RepTable<MAXR> t = {};
+    t.nrep = s.nrep;
+    unsigned off = 0;
+    for (int r = 0; r < s.nrep; ++r) {
+        t.rep[r] = s.reps[r];
+        t.rep[r].dchunks = make_divisor((unsigned)s.reps[r].nx);
+        t.item_off[r] = off;
+        off += (unsigned)(((long long)s.reps[r].nx * s.reps[r].ny * s.reps[r].nz + SEG - 1) / SEG);
+    }
+    t.item_off[s.nrep] = off;
+    return t;
+}
+
 // Launch `kern` on `st`; with `pdl` as the programmatic dependent of the
 // kernel launched before it on that stream (see grid_dependency_wait).
 template <typename... KArgs, typename... Args>
