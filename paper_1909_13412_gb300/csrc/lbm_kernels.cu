@@ -163,6 +163,15 @@ __device__ __forceinline__ void record_sum(unsigned long long rw, int cnt, int x
 // shares.  The block clears the counts of its rows' records of the previous
 // step, which the next step's particle kernel refills.
 // ---------------------------------------------------------------------------
+// Where a segment's mark is compared with the epoch: ahead of the population loads,
+// which then wait for it, or after them.  Which is faster depends on what the
+// compiler makes of the rest: us per step early / late, 256^3 with one particle (and
+// 16777), FP32 rows 1, 2, 4: 347 / 334, 296 / 297 (330 / 333), 341 / 296 (383 / 338);
+// FP16 rows 2: 206 / 216; BF16 rows 1, 2, 4: 241 / 243, 226 / 208 (268 / 265), 220 / 220,
+// and at 255 x 256 x 256 BF16 rows 2 240 / 223.
+template <typename St, int R>
+constexpr bool LATE_MARK = std::is_same<St, StoreF32>::value ? R != 2 : std::is_same<St, StoreBF16>::value && R == 2;
+
 template <int BX, typename St, int R, int MAXR, bool BACK>
 __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
     Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *rec_cur, unsigned long long *rec_prev,
@@ -190,13 +199,19 @@ __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
     NodeIdx n[R];
     float g[R][Q];
     unsigned long long rw[R];
+    unsigned mark[R];
     bool bad = false, forced[R];
 #pragma unroll
     for (int h = 0; h < R; ++h) {
         const unsigned row = grp * R + h < nrows ? grp * R + h : nrows - 1;
         n[h] = node_index(x, row, nx, ny, nz, rp.dny);
         n[h].d += base;
-        forced[h] = mk.epoch == 0 || __ldcg(mk.seg + seg0 + (size_t)row * nchunks + chunk) == mk.epoch;
+        if (LATE_MARK<St, R>) {
+            mark[h] = 0;
+            if (mk.epoch != 0) mark[h] = __ldcg(mk.seg + seg0 + (size_t)row * nchunks + chunk);
+        } else {
+            forced[h] = mk.epoch == 0 || __ldcg(mk.seg + seg0 + (size_t)row * nchunks + chunk) == mk.epoch;
+        }
 #pragma unroll
         for (int a = 0; a < Q; ++a)
             g[h][a] = St::template cload<BACK>(pl.s[a] + (n[h].d + n[h].ox[ex(a) + 1] + n[h].oy[ey(a) + 1] +
@@ -206,7 +221,10 @@ __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
     // (the wait is a no-op unless launched as its programmatic dependent)
     bool wait = blockIdx.x == 0;
 #pragma unroll
-    for (int h = 0; h < R; ++h) wait = wait || forced[h];
+    for (int h = 0; h < R; ++h) {
+        if (LATE_MARK<St, R>) forced[h] = mark[h] == mk.epoch;  // no marks: 0 == 0
+        wait = wait || forced[h];
+    }
     if (wait) grid_dependency_wait();
     grid_dependents_launch();
     if (blockIdx.x == 0 && threadIdx.x == 0) *bump += 1;
@@ -715,9 +733,12 @@ bool lattice_chains(const Sim &s) { return s.variant == 0 || s.variant == 3; }
 // Marks let the segments without forces collide beside the particle kernel.
 // That pays once the pass has more row segments than are resident at a time: below,
 // all already wait with their loads done, and the particle kernel only loses issue
-// slots to them (11.1 -> 11.3 us at 32^3).
+// slots to them (11.1 -> 11.3 us at 32^3).  With FP32 and one row a block it only pays
+// while the buffers are about the size of L2 (with / without, one particle: 26.7 / 31.8
+// at 112^3, 38.3 / 43.3 at 128^3, 69.1 / 65.5 at 144^3, 334 / 305 at 256^3).
 bool lattice_marks(const Sim &s) {
     if (!lattice_chains(s) || s.np == 0) return false;
+    if (s.precision == LBP_F32 && s.rows == 1 && !sweeps_back(s)) return false;
     long long items = 0;  // blocks of the one-node kernel, warps of the four-node one
     for (int r = 0; r < s.nrep; ++r)
         items += ((long long)s.reps[r].ny * s.reps[r].nz + s.rows - 1) / s.rows * s.reps[r].nchunks;

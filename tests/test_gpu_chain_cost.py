@@ -1,0 +1,41 @@
+"""Launching the steps of one call as a chain never costs time, whatever the kernel's shape."""
+import time
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_1909_13412_gb300 import lbp  # noqa: E402
+from paper_1909_13412_gb300 import workloads as wl  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+L = 200  # buffers well beyond L2
+
+
+def step_seconds(h, steps=40):
+    lbp.lbp_step(h, steps)
+    took = []
+    for _ in range(7):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        lbp.lbp_step(h, steps)
+        torch.cuda.synchronize()
+        took.append(time.perf_counter() - t)
+    return float(np.median(took)) / steps
+
+
+@pytest.mark.parametrize("n", [1, 8000])
+@pytest.mark.parametrize("precision,shape", [(lbp.LBP_F32, (r, 0)) for r in (1, 2, 4)] + [(lbp.LBP_BF16, (r, 0)) for r in (1, 2, 4)])
+def test_chain_is_not_slower_than_plain_launches(precision, shape, n):
+    """Within 5 % (two runs of one shape differ by less than 2 %); the marks cost
+    9 to 12 % here with one or four FP32 rows a block."""
+    h = lbp.lbp_create(L, L, L, 0.8, precision=precision)
+    ps = wl.uniform_particles(n, (L, L, L), 10.0, 0.5, 0.26, 1e-4, 5, 6)
+    lbp.lbp_particles_add(h, ps.r, ps.V, ps.M, ps.gamma, ps.R)
+    lbp.lbp_particles_set_params(h, kT=1e-4, seed=3)
+    lbp.lbp_set_block_shape(h, *shape)
+    chain = step_seconds(h)
+    lbp.lbp_set_use_graphs(h, False)
+    assert chain <= 1.05 * step_seconds(h)
+    lbp.lbp_destroy(h)
