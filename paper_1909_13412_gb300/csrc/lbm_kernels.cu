@@ -456,7 +456,10 @@ __device__ __forceinline__ void record_sum4(unsigned long long rw, int cnt, int 
 // Per node the arithmetic is that of collide_st, and the force sums are
 // the same exact integer sums: results equal the other kernels' bit for bit.
 // ---------------------------------------------------------------------------
-constexpr int QUAD_WARPS = 2;  // row segments (warps) per block
+// Row segments (warps) per block.  With several rows a block of four: us per step at
+// 256^3 with 16777 particles, BF16, blocks of two / four: two rows 308 / 299, four rows
+// 551 / 456 (the same within 1 % with one particle); one row: see below.
+constexpr int quad_warps(int R) { return R == 1 ? 2 : 4; }
 // With one row the kernel is bound by latency and instruction issue: it is held
 // to 72 registers for 28 warps per SM.  us a step at 256^3 with 16384 particles,
 // BF16 / FP16: 24 warps (80 registers) 206.5 / 222.0, 28 in blocks of four
@@ -470,11 +473,11 @@ constexpr int QUAD_WARPS = 2;  // row segments (warps) per block
 // flight and need the registers.
 
 template <typename St, int R, int MAXR, bool FORCED, bool BACK>
-__global__ void __launch_bounds__(32 * QUAD_WARPS, R == 1 ? 14 : 1) k_stream_collide_quad(
+__global__ void __launch_bounds__(32 * quad_warps(R), R == 1 ? 14 : 1) k_stream_collide_quad(
     Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *rec_cur,
     unsigned long long *rec_prev, unsigned long long *fq, long long Ntot, long long *bump, int *err, const Marks mk, bool flip) {
     if (!FORCED && blockIdx.x == 0 && threadIdx.x == 0) *bump += 1;
-    const unsigned item = block_of<BACK>(flip) * QUAD_WARPS + (threadIdx.x >> 5);
+    const unsigned item = block_of<BACK>(flip) * quad_warps(R) + (threadIdx.x >> 5);
     if (item >= rt.item_off[MAXR == 1 ? 1 : rt.nrep]) return;  // whole warp past the last segment
     const int r = find_block_rep(rt, item);
     const Rep &rp = rt.rep[r];
@@ -735,13 +738,16 @@ bool lattice_chains(const Sim &s) { return s.variant == 0 || s.variant == 3; }
 // all already wait with their loads done, and the particle kernel only loses issue
 // slots to them (11.1 -> 11.3 us at 32^3).  With FP32 and one row a block it only pays
 // while the buffers are about the size of L2 (with / without, one particle: 26.7 / 31.8
-// at 112^3, 38.3 / 43.3 at 128^3, 69.1 / 65.5 at 144^3, 334 / 305 at 256^3).
+// at 112^3, 38.3 / 43.3 at 128^3, 69.1 / 65.5 at 144^3, 334 / 305 at 256^3), and with
+// four rows in the four-node kernel while most groups of rows stay unmarked, a particle
+// marking four rows (256^3 BF16: 202 / 217 with one particle, 493 / 456 with 16777).
 bool lattice_marks(const Sim &s) {
     if (!lattice_chains(s) || s.np == 0) return false;
     if (s.precision == LBP_F32 && s.rows == 1 && !sweeps_back(s)) return false;
     long long items = 0;  // blocks of the one-node kernel, warps of the four-node one
     for (int r = 0; r < s.nrep; ++r)
         items += ((long long)s.reps[r].ny * s.reps[r].nz + s.rows - 1) / s.rows * s.reps[r].nchunks;
+    if (s.variant == 3 && s.rows == 4 && 4ll * s.np > items) return false;
     return items > (s.variant == 0 ? 8ll : 28ll) * s.num_sms;
 }
 
@@ -807,9 +813,9 @@ static cudaError_t launch_sc(Sim &s, const void *src, void *dst, const unsigned 
                         return launch_k(k_stream_collide_pair<St, R, MAXR, FORCED>, grid, PAIR_BX, 0, st, pdl,
                                         planes_of<St>(s, src, dst), rt, rec_cur, rec_prev, s.fq, s.N, bump, s.d_err);
                     if (use_quad)
-                        return launch_k(k_stream_collide_quad<St, R, MAXR, FORCED, BACK && R == 1>, (grid + QUAD_WARPS - 1) / QUAD_WARPS,
-                                        32 * QUAD_WARPS, 0, st, pdl, planes_of<St>(s, src, dst), rt, rec_cur, rec_prev,
-                                        s.fq, s.N, bump, s.d_err, mk, flip);
+                        return launch_k(k_stream_collide_quad<St, R, MAXR, FORCED, BACK && R == 1>,
+                                        (grid + quad_warps(R) - 1) / quad_warps(R), 32 * quad_warps(R), 0, st, pdl,
+                                        planes_of<St>(s, src, dst), rt, rec_cur, rec_prev, s.fq, s.N, bump, s.d_err, mk, flip);
                 }
                 if constexpr (FORCED)
                     return launch_k(k_stream_collide_forced<BX, St, R, MAXR, BACK>, grid, BX, 0, st, pdl,

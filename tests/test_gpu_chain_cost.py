@@ -26,10 +26,12 @@ def step_seconds(h, steps=40):
 
 
 @pytest.mark.parametrize("n", [1, 8000])
-@pytest.mark.parametrize("precision,shape", [(lbp.LBP_F32, (r, 0)) for r in (1, 2, 4)] + [(lbp.LBP_BF16, (r, 0)) for r in (1, 2, 4)])
+@pytest.mark.parametrize("precision,shape", [(lbp.LBP_F32, (r, 0)) for r in (1, 2, 4)] + [
+    (lbp.LBP_BF16, (r, v)) for v in (0, 3) for r in (1, 2, 4)])
 def test_chain_is_not_slower_than_plain_launches(precision, shape, n):
     """Within 5 % (two runs of one shape differ by less than 2 %); the marks cost
-    9 to 12 % here with one or four FP32 rows a block."""
+    9 to 12 % here with one or four FP32 rows a block, and with four rows of the
+    four-node kernel between many particles."""
     h = lbp.lbp_create(L, L, L, 0.8, precision=precision)
     ps = wl.uniform_particles(n, (L, L, L), 10.0, 0.5, 0.26, 1e-4, 5, 6)
     lbp.lbp_particles_add(h, ps.r, ps.V, ps.M, ps.gamma, ps.R)
