@@ -496,7 +496,7 @@ cudaError_t launch_particles(Sim &s, const void *src, int parity, cudaStream_t s
     A.ring_cap = s.vacf_cap;
     A.d_vacf = s.d_vacf;
     A.err = s.d_err;
-    A.inj = s.inj;
+    A.inj = replay ? nullptr : s.inj;  // the recording has counted these steps
     A.fext_in = io ? io->fext_in : nullptr;
     A.r_out = io ? io->r_out : nullptr;
     A.v_out = io ? io->v_out : nullptr;

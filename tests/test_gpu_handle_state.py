@@ -1,0 +1,47 @@
+"""What calls other than steps leave of a handle's state."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_1909_13412_gb300 import lbp  # noqa: E402
+from paper_1909_13412_gb300 import workloads as wl  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def handle(shape, n, precision=lbp.LBP_F32, stream=None, kT=1e-4):
+    nx, ny, nz = shape
+    h = lbp.lbp_create(nx, ny, nz, 0.8, precision=precision, stream=stream)
+    if n:
+        ps = wl.uniform_particles(n, (nz, ny, nx), 10.0, 0.5, 0.26, 1e-3, 5, 6)
+        lbp.lbp_particles_add(h, ps.r, ps.V * 30, ps.M, ps.gamma, ps.R)
+        lbp.lbp_particles_set_params(h, kT=kT, seed=3)
+    return h
+
+
+def state(h):
+    n = h.np
+    out = [np.empty((15, h.N))] + [np.empty((n, 3)) for _ in range(4)]
+    lbp.lbp_read_populations(h, out[0])
+    if n:
+        lbp.lbp_particles_read(h, *out[1:])
+    return out
+
+
+def same(a, b):
+    return len(a) == len(b) and all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("chain", [True, False])
+def test_backward_leaves_the_conservation_budget(chain):
+    """The reverse sweep replays the recorded steps: what F_R and F_ext put in was
+    counted when they were recorded."""
+    h = handle((20, 18, 16), 30)
+    lbp.lbp_set_use_graphs(h, chain)
+    lbp.lbp_particles_set_external_force(h, np.full((30, 3), 1e-5))
+    lbp.lbp_budget_track(h)
+    lbp.lbp_adjoint_record(h, 12, 5)
+    before = lbp.lbp_budget(h)
+    lbp.lbp_adjoint_backward(h, 12, np.ones((12, 30, 3)), None, {"v0": np.empty((30, 3))})
+    assert np.array_equal(lbp.lbp_budget(h), before) and before[7:].any()
+    lbp.lbp_destroy(h)
