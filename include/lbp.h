@@ -40,6 +40,9 @@
  * the stream given to lbp_create, and later work on that stream is ordered
  * after it.  Calls that take host pointers return after their copies finish;
  * calls that take device pointers are asynchronous with respect to the host.
+ * Steps cannot be captured into a CUDA graph: while that stream is being
+ * captured, lbp_step, lbp_step_exchange, lbp_autotune and the lbp_adjoint calls
+ * return LBP_ESTATE and leave both the handle and the capture as they were.
  * A handle must not be used from two host threads at once.
  *
  * Errors: every call returns an lbp_status; nothing is thrown across the ABI.

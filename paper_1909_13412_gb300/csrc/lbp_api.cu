@@ -97,6 +97,16 @@ lbp_status leave(lbp_sim *s) {
     return LBP_OK;
 }
 
+// Steps are not recorded into a CUDA graph of the caller's: which of the two
+// population buffers is current and the step index are kept on the host, where a
+// replay does not advance them.  Checked before anything joins the capture.
+lbp_status not_captured(lbp_sim *s, const char *call) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s->user, &st));
+    if (st == cudaStreamCaptureStatusNone) return LBP_OK;
+    return fail(LBP_ESTATE, "%s: the handle's stream is being captured into a CUDA graph", call);
+}
+
 void free_work(lbp_sim *s) {
     if (s->work_mem) cudaFree(s->work_mem);
     s->work_mem = nullptr;
@@ -965,6 +975,7 @@ lbp_status lbp_step(lbp_sim *s, int64_t nsteps) {
     CHECK_SIM(s);
     if (nsteps < 0) return fail(LBP_EINVAL, "lbp_step: nsteps < 0");
     if (nsteps == 0) return LBP_OK;
+    TRY(not_captured(s, "lbp_step"));
     TRY(enter(s));
     Chain c{nsteps};
     for (int64_t n = 0; n < nsteps; ++n) TRY(step_once(s, c));
@@ -975,6 +986,7 @@ lbp_status lbp_step(lbp_sim *s, int64_t nsteps) {
 lbp_status lbp_step_exchange(lbp_sim *s, const double *f_ext, double *r, double *v, int on_device) {
     Range range("lbp_step_exchange");
     CHECK_SIM(s);
+    TRY(not_captured(s, "lbp_step_exchange"));
     TRY(enter(s));
     const int n = s->np;
     if (n > 0 && (f_ext || r || v)) {
@@ -1199,6 +1211,7 @@ lbp_status lbp_autotune(lbp_sim *s, int launches, int *rows, int *variant, doubl
     Range range("lbp_autotune");
     CHECK_SIM(s);
     if (launches < 1 || launches > 1000) return fail(LBP_EINVAL, "lbp_autotune: launches must be in [1, 1000]");
+    TRY(not_captured(s, "lbp_autotune"));
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
     // candidates k = 0..9: (variant, rows) = (0: 1, 2, 4 rows), (1: 1, 2, 4),
@@ -1276,6 +1289,7 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     if (nsteps < 1 || checkpoint_every < 1)
         return fail(LBP_EINVAL, "lbp_adjoint_record: need nsteps >= 1 and checkpoint_every >= 1");
     if (s->np < 1) return fail(LBP_ESTATE, "lbp_adjoint_record: add particles first (the recorded outputs are their trajectories)");
+    TRY(not_captured(s, "lbp_adjoint_record"));
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
     s->tape = lbp::Tape();  // a new recording replaces the previous one
@@ -1338,6 +1352,7 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
     if (tp.T == 0) return fail(LBP_ESTATE, "lbp_adjoint_backward: nothing recorded (lbp_adjoint_record)");
     if (s->step != tp.step0 + tp.T || s->edits != tp.edits || s->np != tp.np)
         return fail(LBP_ESTATE, "lbp_adjoint_backward: the handle changed since lbp_adjoint_record");
+    TRY(not_captured(s, "lbp_adjoint_backward"));
     TRY(enter(s));
     CK(cudaStreamSynchronize(s->s0));
     const int np = s->np, cap = s->cap > 0 ? s->cap : 1, C = tp.C;

@@ -45,3 +45,40 @@ def test_backward_leaves_the_conservation_budget(chain):
     lbp.lbp_adjoint_backward(h, 12, np.ones((12, 30, 3)), None, {"v0": np.empty((30, 3))})
     assert np.array_equal(lbp.lbp_budget(h), before) and before[7:].any()
     lbp.lbp_destroy(h)
+
+
+@pytest.mark.parametrize("warm", [0, 3])
+@pytest.mark.parametrize("n", [0, 5])
+def test_steps_refuse_to_be_captured(n, warm):
+    """A replay would not advance the host's buffer parity and step index.  The
+    capture itself stays valid, and the handle goes on as if not called."""
+    st = torch.cuda.Stream()
+    h, twin = (handle((24, 16, 12), n, stream=s) for s in (st, None))
+    for k in (h, twin):
+        if warm:
+            lbp.lbp_step(k, warm)
+    x = torch.zeros(4, device="cuda")
+    v = torch.empty((3, n, 3), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    calls = [lambda: lbp.lbp_step(h, 1), lambda: lbp.lbp_step(h, 2), lambda: lbp.lbp_step_exchange(h),
+             lambda: lbp.lbp_autotune(h, 1)]
+    if n:
+        calls += [lambda: lbp.lbp_adjoint_record(h, 3, 1, v), lambda: lbp.lbp_step_exchange(h, v[0], v[1], v[2])]
+    with torch.cuda.graph(g, stream=st):
+        x.add_(1)
+        for call in calls:
+            with pytest.raises(lbp.LbpError) as ei:
+                call()
+            assert ei.value.status == lbp.LBP_ESTATE
+        lbp.lbp_step(h, 0)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [3.0] * 4
+    for k in (h, twin):
+        lbp.lbp_step(k, 4)
+    assert lbp.lbp_get_step_index(h) == warm + 4
+    assert same(state(h), state(twin))
+    lbp.lbp_destroy(h)
+    lbp.lbp_destroy(twin)
