@@ -362,15 +362,20 @@ lbp_status lbp_set_body_force(lbp_sim *sim, int replica, const double *g);
  *              stores, one warp per 128-node row segment, 1, 2 or 4 rows
  *              (2-byte storage, every box's nx a multiple of 4).
  * Each candidate runs `launches` back-to-back launches (1..1000) after two
- * warm-up launches, twice, best pass kept.  rows, variant (optional) receive
- * the pick; ms (optional, LBP_AUTOTUNE_CANDIDATES doubles) the mean launch
- * times in ms for (variant 0: 1, 2, 4 rows; variant 1: 1, 2, 4 rows;
- * variant 2; variant 3: 1, 2, 4 rows), -1 where a candidate does not apply.
+ * warm-up launches, twice, best pass kept.  Steps of variants 1 and 2 are not
+ * launched as a chain (lbp_set_use_graphs): a candidate of these that is as fast
+ * alone as the fastest of variants 0 and 3 goes by whole steps, `launches` of
+ * them timed the same way, and its time is that one's plus what its step takes
+ * more.  rows, variant (optional) receive the pick; ms (optional,
+ * LBP_AUTOTUNE_CANDIDATES doubles) the times in ms of (variant 0: 1, 2, 4 rows;
+ * variant 1: 1, 2, 4 rows; variant 2; variant 3: 1, 2, 4 rows), -1 where a
+ * candidate does not apply.
  * The simulation state is unchanged: the launches read the current
  * populations, write only the buffer the next step overwrites, read a copy of
  * the last step's force records (all zero before the first step; run a few
  * steps first for timings that include the particle coupling) and bump a
- * scratch step counter.
+ * scratch step counter; the steps keep records, particle state and step index
+ * in scratch memory of their own.
  * Synchronous; LBP_ETIMEOUT if a bounded device wait ran out.  Default before
  * any call (the picks measured at 256^3): variant 0 with 2 rows for LBP_F32;
  * variant 3 with 1 row for the 2-byte types when every box's nx is a multiple

@@ -1207,6 +1207,79 @@ lbp_status lbp_set_block_rows(lbp_sim *s, int rows) {
     return lbp_set_block_shape(s, rows, s->variant == 2 ? 0 : s->variant);
 }
 
+}  // extern "C"
+
+namespace {
+
+// ms per step of the current block shape, launched as lbp_step launches them, of
+// steps that leave the handle as it is: they read the current populations and write
+// the buffer the next step overwrites, and records, step index and particle state
+// are in `mem` (step_scratch bytes, as the adjoint's replay keeps its own).
+size_t step_scratch(const lbp_sim *s) {
+    return sizeof(long long) * 3 +
+           (s->np > 0 ? sizeof(unsigned long long) * 2 * REC_WORDS * (size_t)s->nseg + sizeof(double) * 12 * s->cap : 0);
+}
+
+cudaError_t time_steps(lbp_sim *s, int steps, void *mem, cudaEvent_t e0, cudaEvent_t e1, double *ms) {
+    const size_t words = s->np > 0 ? (size_t)s->nseg * REC_WORDS : 0, plane = (size_t)3 * s->cap;
+    unsigned long long *rec = static_cast<unsigned long long *>(mem);
+    double *state = reinterpret_cast<double *>(rec + 2 * words);  // [12][cap]: read from, written to
+    long long *step = reinterpret_cast<long long *>(state + (s->np > 0 ? 4 * plane : 0));
+    cudaError_t e = cudaMemsetAsync(rec, 0, sizeof(*rec) * 2 * words, s->s0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(step, s->d_step, sizeof(*step), cudaMemcpyDeviceToDevice, s->s0);
+    if (s->np > 0) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(state, s->r, sizeof(double) * plane, cudaMemcpyDeviceToDevice, s->s0);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(state + plane, s->v, sizeof(double) * plane, cudaMemcpyDeviceToDevice, s->s0);
+    }
+    long long *const saved_step = s->d_step;
+    unsigned long long *const saved_rec[2] = {s->rec[0], s->rec[1]};
+    const int saved_lag = s->vacf_lag;
+    s->d_step = step;
+    s->vacf_lag = -1;  // no samples
+    if (s->np > 0) {
+        s->rec[0] = rec;
+        s->rec[1] = rec + words;
+    }
+    const void *src = s->f[s->cur];
+    void *dst = s->f[s->cur ^ 1];
+    const ParticleIO io{nullptr, nullptr, nullptr, false, state, state + 2 * plane};
+    const bool chains = s->chain && lattice_chains(*s);
+    auto run = [&](int count) {
+        unsigned epoch = 0;
+        for (int i = 0; i < count && e == cudaSuccess; ++i) {
+            const unsigned next = i + 1 < count && s->chain && lattice_marks(*s) ? ++s->epoch : 0;
+            if (s->np > 0) {
+                e = launch_particles(*s, src, i & 1, s->s0, &io, i > 0 && chains, next);
+                if (e == cudaSuccess) e = launch_stream_collide_forced(*s, src, dst, i & 1, s->s0, true, epoch);
+            } else {
+                e = launch_stream_collide(*s, src, dst, i & 1, s->s0, i > 0 && chains);
+            }
+            epoch = next;
+        }
+    };
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        run(2);
+        if (e == cudaSuccess) e = cudaEventRecord(e0, s->s0);
+        run(steps);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, s->s0);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float el = 0.f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&el, e0, e1);
+        const double per = (double)el / steps;
+        *ms = pass == 0 ? per : std::min(*ms, per);
+    }
+    s->d_step = saved_step;
+    s->vacf_lag = saved_lag;
+    s->rec[0] = saved_rec[0];
+    s->rec[1] = saved_rec[1];
+    return e;
+}
+
+}  // namespace
+
+extern "C" {
+
 lbp_status lbp_autotune(lbp_sim *s, int launches, int *rows, int *variant, double *ms) {
     Range range("lbp_autotune");
     CHECK_SIM(s);
@@ -1262,13 +1335,55 @@ lbp_status lbp_autotune(lbp_sim *s, int launches, int *rows, int *variant, doubl
             const double per = (double)el / launches;
             if (e == cudaSuccess) t[k] = pass == 0 ? per : std::min(t[k], per);
         }
+    // a variant whose steps are not chained and that is as fast alone as the fastest
+    // that chains goes by its steps: its time is that one's plus what its step takes more
+    auto chains = [&](int k) { return cand_v[k] == 0 || cand_v[k] == 3; };
+    int ref = 0;  // variant 0 always applies
+    for (int k = 0; k < NC; ++k)
+        if (chains(k) && t[k] > 0 && t[k] < t[ref]) ref = k;
+    int err = 0;
+    if (e == cudaSuccess) e = cudaMemcpy(&err, s->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && !(err & ERR_TIMEOUT) && s->chain) {
+        const int saved_rows = s->rows, saved_variant = s->variant, before = err;
+        void *mem = nullptr;
+        double ref_step = 0.0, step = 0.0;
+        auto steps_of = [&](int k, double *ms_step) {
+            s->rows = cand_r[k];
+            s->variant = cand_v[k];
+            if (e == cudaSuccess) e = time_steps(s, launches, mem, e0, e1, ms_step);
+        };
+        for (int k = 0; k < NC && e == cudaSuccess; ++k) {
+            if (chains(k) || !(t[k] > 0) || t[k] > t[ref]) continue;
+            if (!mem) {
+                if (cudaMalloc(&mem, step_scratch(s)) != cudaSuccess) {  // they stay at their times alone
+                    (void)cudaGetLastError();
+                    mem = nullptr;
+                    break;
+                }
+                steps_of(ref, &ref_step);
+            }
+            steps_of(k, &step);
+            t[k] = std::max(t[ref] + step - ref_step, 1e-6);
+        }
+        s->rows = saved_rows;
+        s->variant = saved_variant;
+        if (mem) {
+            if (e == cudaSuccess) e = cudaMemcpy(&err, s->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+            if (err & ERR_TIMEOUT) {
+                // a pass that gave up left its overflow shares
+                if (s->fq) cudaMemset(s->fq, 0, sizeof(unsigned long long) * 3 * (size_t)s->N);
+            } else if (e == cudaSuccess && err != before) {
+                // what these steps would report, the handle's own will
+                e = cudaMemcpy(s->d_err, &before, sizeof(int), cudaMemcpyHostToDevice);
+            }
+            cudaFree(mem);
+        }
+    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(scr);
     if (e != cudaSuccess) return fail(LBP_ECUDA, "lbp_autotune: %s", cudaGetErrorString(e));
     // a bounded wait inside the staged kernel that ran out shows in the error flag
-    int err = 0;
-    CK(cudaMemcpy(&err, s->d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (err & ERR_TIMEOUT) return fail(LBP_ETIMEOUT, "lbp_autotune: a bounded wait in the staged kernel ran out");
     int best = -1;
     for (int k = 0; k < NC; ++k)

@@ -1,4 +1,6 @@
 """What calls other than steps leave of a handle's state."""
+import time
+
 import numpy as np
 import pytest
 
@@ -82,3 +84,63 @@ def test_steps_refuse_to_be_captured(n, warm):
     assert same(state(h), state(twin))
     lbp.lbp_destroy(h)
     lbp.lbp_destroy(twin)
+
+
+def step_seconds(h, steps=60):
+    lbp.lbp_step(h, steps)
+    took = []
+    for _ in range(5):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        lbp.lbp_step(h, steps)
+        torch.cuda.synchronize()
+        took.append(time.perf_counter() - t)
+    return float(np.median(took)) / steps
+
+
+@pytest.mark.parametrize("shape,n", [((66, 64, 64), 0), ((34, 32, 32), 1), ((62, 66, 60), 0), ((126, 128, 128), 500)])
+@pytest.mark.parametrize("precision", [lbp.LBP_BF16, lbp.LBP_F16])
+def test_autotune_picks_the_fastest_step(shape, n, precision):
+    """Boxes where the two-node kernel, whose steps are not chained, is as fast as
+    the others alone: every pick's step within 15 % of the best one's (the steps
+    differ by 20 to 50 % there)."""
+    h = handle(shape, n, precision)
+    lbp.lbp_step(h, 3)
+    picks = {lbp.lbp_autotune(h, 5)[:2] for _ in range(12)}
+    took = {}
+    for rows, variant in [(1, 0), (2, 0), (4, 0), (1, 1), (2, 1)]:
+        lbp.lbp_set_block_shape(h, rows, variant)
+        took[rows, variant] = step_seconds(h)
+    for pick in picks:
+        assert took.get(pick, np.inf) <= 1.15 * min(took.values()), (pick, took)
+    lbp.lbp_destroy(h)
+
+
+@pytest.mark.parametrize("shape,n,precision", [((66, 24, 20), 0, lbp.LBP_F16), ((34, 32, 32), 40, lbp.LBP_BF16), ((62, 20, 24), 2, lbp.LBP_F16),
+                                               ((3, 5, 130), 60, lbp.LBP_F32), ((32, 24, 16), 9, lbp.LBP_F32)])
+def test_autotune_leaves_the_handle(shape, n, precision):
+    """Also where whole steps are timed: a tuned handle goes on as its twin, with the
+    correlator, the conservation budget and the error flag as they were."""
+    out = []
+    for tune in (True, False):
+        h = handle(shape, n, precision)
+        lbp.lbp_budget_track(h)
+        if n:
+            lbp.lbp_vacf_configure(h, 20)
+        lbp.lbp_step(h, 7)
+        before = lbp.lbp_budget(h), lbp.lbp_diagnostics(h)["overflow_shares"], lbp.lbp_get_step_index(h)
+        if tune:
+            for _ in range(8):
+                lbp.lbp_autotune(h, 3)
+                after = lbp.lbp_budget(h), lbp.lbp_diagnostics(h)["overflow_shares"], lbp.lbp_get_step_index(h)
+                assert np.array_equal(before[0], after[0]) and before[1:] == after[1:]
+        lbp.lbp_check(h)
+        lbp.lbp_step(h, 80)
+        res = state(h)
+        if n:
+            res += [np.empty(21), np.empty(21, np.int64)]
+            lbp.lbp_vacf_read(h, *res[-2:])
+        lbp.lbp_check(h)
+        lbp.lbp_destroy(h)
+        out.append(res)
+    assert same(*out)
