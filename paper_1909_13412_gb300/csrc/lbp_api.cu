@@ -279,20 +279,10 @@ lbp_status exchange_out(lbp_sim *s, double *r, double *v, cudaMemcpyKind kind, c
     return LBP_OK;
 }
 
-// the device address of a mapped page-locked host buffer (null stays null)
-lbp_status device_view(double *&p) {
-    if (!p) return LBP_OK;
-    cudaPointerAttributes at;
-    CK(cudaPointerGetAttributes(&at, p));
-    p = static_cast<double *>(at.devicePointer);
-    return LBP_OK;
-}
-
-// one step whose particle kernel reads the forces from, and writes positions and
-// velocities to, page-locked host buffers or device buffers
-lbp_status exchange_step(lbp_sim *s, const double *f_ext, double *r, double *v, int on_device) {
-    double *f_dev = const_cast<double *>(f_ext), *r_dev = r, *v_dev = v;
-    if (!on_device) {
+// one step whose particle kernel does the exchange's I/O itself (io: from
+// kernel_view); for page-locked host buffers it raises the completion flag
+lbp_status exchange_step(lbp_sim *s, const ParticleIO &io) {
+    if (io.signal) {
         if (!s->d_xticket) {
             TRY(dalloc(&s->d_xticket, 1));
             CK(cudaMemsetAsync(s->d_xticket, 0, sizeof(unsigned), s->s0));
@@ -301,14 +291,10 @@ lbp_status exchange_step(lbp_sim *s, const double *f_ext, double *r, double *v, 
             CK(cudaHostAlloc((void **)&s->h_xflag, sizeof(long long), cudaHostAllocMapped));
             CK(cudaHostGetDevicePointer((void **)&s->h_xflag_dev, s->h_xflag, 0));
         }
-        TRY(device_view(f_dev));
-        TRY(device_view(r_dev));
-        TRY(device_view(v_dev));
         // the flag may hold this step index from before a lbp_set_step_index or a
         // checkpoint load; the previous call's kernel has finished writing it
         __atomic_store_n(s->h_xflag, -1ll, __ATOMIC_RELEASE);
     }
-    const ParticleIO io{f_dev, r_dev, v_dev, !on_device};
     Chain c{1};
     return step_once(s, c, &io);
 }
@@ -334,32 +320,27 @@ lbp_status wait_exchange_flag(lbp_sim *s, long long step) {
     }
 }
 
-// page-locked (or registered) host memory mapped into the device's address
-// space, which kernels can read and write directly (FP64 elements: 8-byte
-// aligned; anything else takes the copies, which accept any alignment)
-bool host_pinned(const void *p) {
-    if (!p) return true;
-    if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeHost && at.devicePointer != nullptr;
-}
-
-// memory of the current device that its kernels can read and write directly
-// (8-byte aligned, as host_pinned)
-bool device_memory(const void *p) {
+// The address at which kernels can read and write a caller's FP64 buffer directly
+// (null stays null): page-locked (or registered) host memory mapped into the
+// device's address space, or memory of the current device.  False for anything
+// else, and for addresses that are not 8-byte aligned: those take the copies,
+// which accept any.  One query a buffer, as an exchange call makes three.
+bool kernel_view(const double *p, int on_device, double **view) {
+    *view = nullptr;
     if (!p) return true;
     if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
     int dev = 0;
     cudaPointerAttributes at;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || (on_device && cudaGetDevice(&dev) != cudaSuccess)) {
         cudaGetLastError();
         return false;
     }
-    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == dev;
+    if (on_device) {
+        *view = const_cast<double *>(p);
+        return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == dev;
+    }
+    *view = static_cast<double *>(at.devicePointer);
+    return at.type == cudaMemoryTypeHost && at.devicePointer != nullptr;
 }
 
 
@@ -1000,12 +981,12 @@ lbp_status lbp_step_exchange(lbp_sim *s, const double *f_ext, double *r, double 
         }
     }
     if (n > 0 && f_ext) s->edits += 1;  // as lbp_particles_set_external_force
-    const bool direct = n > 0 && !s->timing &&
-                        (on_device ? device_memory(f_ext) && device_memory(r) && device_memory(v)
-                                   : host_pinned(f_ext) && host_pinned(r) && host_pinned(v));
+    double *f_dev = nullptr, *r_dev = nullptr, *v_dev = nullptr;
+    const bool direct = n > 0 && !s->timing && kernel_view(f_ext, on_device, &f_dev) &&
+                        kernel_view(r, on_device, &r_dev) && kernel_view(v, on_device, &v_dev);
     if (direct) {
         const long long step = s->step;
-        TRY(exchange_step(s, f_ext, r, v, on_device));
+        TRY(exchange_step(s, ParticleIO{f_dev, r_dev, v_dev, !on_device}));
         // host buffers: return once f_ext has been consumed and r, v are on the
         // host; the step's lattice pass may still run, and later work on s0
         // follows it.  Device buffers: stream-ordered like any other step.

@@ -105,3 +105,11 @@ def test_force_overflow_is_read_through_l2(name, file):
     reads = [r for r in reads if not re.search(r"\bfqd?\s*\[[^=]*\]\s*=[^=]", r)]
     assert reads or "__ldcg(fq" in body
     assert all("__ldcg(fq" in r for r in reads), reads
+
+
+def test_exchange_asks_for_a_buffers_attributes_once():
+    """Each of an exchange call's three buffers costs one driver query (about 0.2 us)."""
+    text = source("lbp_api.cu")
+    assert text.count("cudaPointerGetAttributes(") == 1
+    body = block(text, text.index("{", text.index("lbp_status lbp_step_exchange(")))
+    assert body.count("kernel_view(") == 3
