@@ -34,7 +34,8 @@
  * order (particle ids are 0, 1, ... in the order of lbp_particles_add calls).
  *
  * Memory and streams: the library owns its device state (allocated at create
- * and at particles_add).  Every pointer passed in is owned by the caller; it is
+ * and at particles_add; the memory of a gradient, see lbp_adjoint_release, at
+ * the gradient).  Every pointer passed in is owned by the caller; it is
  * a host pointer if the call's on_device argument is 0, else a device pointer
  * on the current device.  All work is ordered after the work already queued on
  * the stream given to lbp_create, and later work on that stream is ordered
@@ -481,6 +482,18 @@ lbp_status lbp_adjoint_record(lbp_sim *sim, int64_t nsteps, int checkpoint_every
                               double *r_traj, int on_device);
 lbp_status lbp_adjoint_backward(lbp_sim *sim, const double *g_v, const double *g_r, int on_device,
                                 const lbp_gradients *grads);
+
+/* Drop the recording and give the memory of the handle's gradients back now:
+ * lbp_adjoint_backward then returns LBP_ESTATE until the next
+ * lbp_adjoint_record.  Otherwise the handle keeps two blocks for its next
+ * gradient, reused while they are large enough and at most twice what is asked:
+ * the recording's, and the reverse sweep's (checkpoint_every - 1 copies of the
+ * populations and two FP32 ones for dL/df).  The sweep's is given back at the
+ * end of lbp_adjoint_backward if the two hold more than an eighth of the
+ * device's memory, or it more than a quarter of what is left free, and when an
+ * allocation of any handle in the process would fail without.  Programs that
+ * need the memory for allocations of their own call this after a gradient.   */
+lbp_status lbp_adjoint_release(lbp_sim *sim);
 
 /* Message of the calling thread's last failing call ("" if none).            */
 const char *lbp_last_error(void);

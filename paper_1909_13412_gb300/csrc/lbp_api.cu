@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <cstring>
 #include <chrono>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -34,6 +35,7 @@ struct lbp_sim : public lbp::Sim {
     std::vector<double> h_gamma, h_radius;  // host copies for parameter updates
     std::vector<double> h_mass;             // host copy for the momentum budget
     std::vector<int> h_prep;                // replica of each particle
+    lbp_sim *next_idle = nullptr;           // list of idle reverse-sweep blocks (g_idle)
 };
 
 namespace {
@@ -107,25 +109,65 @@ lbp_status not_captured(lbp_sim *s, const char *call) {
     return fail(LBP_ESTATE, "%s: the handle's stream is being captured into a CUDA graph", call);
 }
 
+// Handles that keep a reverse sweep's block which no call is using (see
+// adjoint_memory): when an allocation of any handle fails, on any host thread,
+// they give theirs up.  A handle touches its own block only after take_work.
+std::mutex g_idle_mu;
+lbp_sim *g_idle = nullptr;
+
+void take_work(lbp_sim *s) {
+    std::lock_guard<std::mutex> lock(g_idle_mu);
+    for (lbp_sim **p = &g_idle; *p; p = &(*p)->next_idle)
+        if (*p == s) {
+            *p = s->next_idle;
+            return;
+        }
+}
+
+void keep_work(lbp_sim *s) {
+    std::lock_guard<std::mutex> lock(g_idle_mu);
+    s->next_idle = g_idle;
+    g_idle = s;
+}
+
+// of a block that take_work has taken
 void free_work(lbp_sim *s) {
     if (s->work_mem) cudaFree(s->work_mem);
     s->work_mem = nullptr;
     s->work_bytes = 0;
 }
 
-// device memory for the handle, for which it gives up the reverse sweep's block if need be
-lbp_status handle_alloc(lbp_sim *s, void **mem, size_t bytes) {
-    cudaError_t e = cudaMalloc(mem, bytes);
-    if (e == cudaErrorMemoryAllocation && s->work_mem) {
-        (void)cudaGetLastError();
+bool free_idle(int dev) {
+    std::lock_guard<std::mutex> lock(g_idle_mu);
+    bool any = false;
+    for (lbp_sim **p = &g_idle; *p;) {
+        lbp_sim *s = *p;
+        if (s->dev != dev) {
+            p = &s->next_idle;
+            continue;
+        }
+        *p = s->next_idle;
+        any = any || s->work_mem;
         free_work(s);
-        e = cudaMalloc(mem, bytes);
     }
-    if (e == cudaSuccess) return LBP_OK;
-    *mem = nullptr;
-    (void)cudaGetLastError();
-    return fail(e == cudaErrorMemoryAllocation ? LBP_ENOMEM : LBP_ECUDA, "cudaMalloc of %zu bytes: %s", bytes,
-                cudaGetErrorString(e));
+    return any;
+}
+
+cudaError_t device_malloc(void **mem, size_t bytes) {
+    cudaError_t e = cudaMalloc(mem, bytes);
+    int dev = 0;
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        if (cudaGetDevice(&dev) == cudaSuccess && free_idle(dev)) e = cudaMalloc(mem, bytes);
+    }
+    if (e != cudaSuccess) *mem = nullptr;
+    return e;
+}
+
+template <typename T>
+lbp_status dalloc(T **p, size_t count) {
+    CK(device_malloc((void **)p, sizeof(T) * (count ? count : 1)));
+    return LBP_OK;
 }
 
 lbp_status stage(lbp_sim *s, size_t bytes) {
@@ -136,16 +178,8 @@ lbp_status stage(lbp_sim *s, size_t bytes) {
         s->stage = nullptr;
         s->stage_bytes = 0;
     }
-    TRY(handle_alloc(s, (void **)&s->stage, bytes));
+    CK(device_malloc((void **)&s->stage, bytes));
     s->stage_bytes = bytes;
-    return LBP_OK;
-}
-
-template <typename T>
-lbp_status dalloc(T **p, size_t count) {
-    *p = nullptr;
-    if (count == 0) count = 1;
-    CK(cudaMalloc((void **)p, sizeof(T) * count));
     return LBP_OK;
 }
 
@@ -347,15 +381,15 @@ bool kernel_view(const double *p, int on_device, double **view) {
 // The recording's and the reverse sweep's device memory, one block each, kept by
 // the handle: at 256^3 with 10 steps a segment, mapping and unmapping 13 GB took 9
 // of a 35 ms gradient.  A block is reused while it is large enough and not more
-// than twice what is asked; the sweep's is given back at the end of the call when
-// the two would hold more than an eighth of the device's memory, before other
-// large allocations of the handle, and when one of these fails.
-lbp_status adjoint_memory(lbp_sim *s, void **mem, size_t *have, size_t bytes) {
+// than twice what is asked.  The sweep's is given back at the end of the call when
+// the two hold more than an eighth of the device's memory or it more than a quarter
+// of what is left free, when an allocation of any handle fails (free_idle), and by
+// lbp_adjoint_release, as the recording's.
+lbp_status adjoint_memory(void **mem, size_t *have, size_t bytes) {
     if (*mem && *have >= bytes && *have / 2 <= bytes) return LBP_OK;
     if (*mem) cudaFree(*mem);
-    *mem = nullptr;
     *have = 0;
-    TRY(handle_alloc(s, mem, bytes));
+    CK(device_malloc(mem, bytes));
     *have = bytes;
     return LBP_OK;
 }
@@ -519,6 +553,7 @@ lbp_status lbp_destroy(lbp_sim *s) {
     if (!s) return LBP_OK;
     if (s->s0) cudaStreamSynchronize(s->s0);
     if (s->s1) cudaStreamSynchronize(s->s1);
+    take_work(s);
     void *bufs[] = {s->f[0], s->f[1], s->d_step, s->d_err, s->r, s->v, s->fh, s->fr, s->fext, s->xbuf,
                     s->mass, s->inv_mass, s->gamma, s->radius, s->sig, s->pinned, s->prep, s->fq, s->rec[0],
                     s->rec[1], s->marks[0], s->marks[1], s->ring,
@@ -682,7 +717,6 @@ lbp_status lbp_particles_add_to(lbp_sim *s, int replica, int n, const double *r,
     if (np_new > s->cap) {
         int cap = s->cap ? s->cap : 64;
         while (cap < np_new) cap *= 2;
-        free_work(s);
         CK(cudaStreamSynchronize(s->s0));
         CK(cudaStreamSynchronize(s->s1));
         double **vec[] = {&s->r, &s->v, &s->fh, &s->fr, &s->fext};
@@ -1044,7 +1078,6 @@ lbp_status lbp_vacf_configure_ex(lbp_sim *s, int max_lag, int per_particle) {
         }
     if (max_lag < 0) return leave(s);
     if (s->np == 0) return fail(LBP_ESTATE, "lbp_vacf_configure: add particles first");
-    free_work(s);
     const int B = vacf_block_samples();
     const long long ncomp = 3ll * s->np;
     // per particle: FP32 ring of max_lag + 2 blocks (one block more than the
@@ -1336,7 +1369,7 @@ lbp_status lbp_autotune(lbp_sim *s, int launches, int *rows, int *variant, doubl
         for (int k = 0; k < NC && e == cudaSuccess; ++k) {
             if (chains(k) || !(t[k] > 0) || t[k] > t[ref]) continue;
             if (!mem) {
-                if (cudaMalloc(&mem, step_scratch(s)) != cudaSuccess) {  // they stay at their times alone
+                if (device_malloc(&mem, step_scratch(s)) != cudaSuccess) {  // they stay at their times alone
                     (void)cudaGetLastError();
                     mem = nullptr;
                     break;
@@ -1395,7 +1428,7 @@ lbp_status lbp_adjoint_record(lbp_sim *s, int64_t nsteps, int checkpoint_every, 
     const size_t pcount = (size_t)6 * (s->cap > 0 ? s->cap : 1);
     Carve c;
     const size_t at_f = c.add(pop_bytes * (size_t)nck), at_p = c.add(sizeof(double) * pcount * (size_t)nck);
-    TRY(adjoint_memory(s, &s->tape_mem, &s->tape_bytes, c.bytes));
+    TRY(adjoint_memory(&s->tape_mem, &s->tape_bytes, c.bytes));
     tp.ck_f = static_cast<char *>(s->tape_mem) + at_f;
     tp.ck_p = reinterpret_cast<double *>(static_cast<char *>(s->tape_mem) + at_p);
     const size_t traj = (size_t)nsteps * s->np * 3;
@@ -1469,13 +1502,17 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
                  at_lvr = c.add(sizeof(double) * (n_lvr + n_acc + n_om)),
                  at_g = c.add(stage_g ? sizeof(double) * 2 * traj : 0),
                  at_f0 = c.add(out->f0 && !on_device ? sizeof(double) * Q * s->N : 0);  // dL/df0 for a host destination
-    TRY(adjoint_memory(s, &s->work_mem, &s->work_bytes, c.bytes));
-    // given back at the end if it is much
+    take_work(s);
+    TRY(adjoint_memory(&s->work_mem, &s->work_bytes, c.bytes));
     struct Guard {
         lbp_sim *s;
         ~Guard() {
-            size_t free_b = 0, total = 0;
-            if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || s->tape_bytes + s->work_bytes > total / 8) free_work(s);
+            size_t left = 0, total = 0;
+            if (cudaMemGetInfo(&left, &total) != cudaSuccess || s->tape_bytes + s->work_bytes > total / 8 ||
+                s->work_bytes > left / 4)
+                free_work(s);
+            else
+                keep_work(s);
         }
     } guard{s};
     char *work = static_cast<char *>(s->work_mem);
@@ -1633,6 +1670,18 @@ lbp_status lbp_adjoint_backward(lbp_sim *s, const double *g_v, const double *g_r
     restore();
     if (st != LBP_OK) return st;
     return leave(s);
+}
+
+lbp_status lbp_adjoint_release(lbp_sim *s) {
+    CHECK_SIM(s);
+    CK(cudaStreamSynchronize(s->s0));
+    s->tape = lbp::Tape();
+    take_work(s);
+    free_work(s);
+    if (s->tape_mem) cudaFree(s->tape_mem);
+    s->tape_mem = nullptr;
+    s->tape_bytes = 0;
+    return LBP_OK;
 }
 
 lbp_status lbp_check(lbp_sim *s) {

@@ -74,6 +74,7 @@ _SIGS = {
     "lbp_step_exchange": [_vp, _vp, _vp, _vp, C.c_int],
     "lbp_adjoint_record": [_vp, C.c_int64, C.c_int, _vp, _vp, C.c_int],
     "lbp_adjoint_backward": [_vp, _vp, _vp, C.c_int, _vp],
+    "lbp_adjoint_release": [_vp],
     "lbp_set_block_rows": [_vp, C.c_int],
     "lbp_set_body_force": [_vp, C.c_int, _vp],
     "lbp_set_fluid": [_vp, _vp, _vp, C.c_int],
@@ -440,6 +441,11 @@ def lbp_adjoint_backward(h: Handle, nsteps, g_v=None, g_r=None, out=None):
     d = _same_side(a, b, *ptrs)
     _call("lbp_adjoint_backward", h.ptr, a[0], b[0], d, C.byref(g))
     return out
+
+
+def lbp_adjoint_release(h: Handle):
+    """Drop the recording and give the memory of the handle's gradients back."""
+    _call("lbp_adjoint_release", h.ptr)
 
 
 def lbp_check(h: Handle):

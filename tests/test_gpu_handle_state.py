@@ -144,3 +144,67 @@ def test_autotune_leaves_the_handle(shape, n, precision):
         lbp.lbp_destroy(h)
         out.append(res)
     assert same(*out)
+
+
+def gradient(h, steps, every, precision=lbp.LBP_F32):
+    n = h.np
+    lbp.lbp_adjoint_record(h, steps, every)
+    g = np.random.default_rng(1).standard_normal((steps, n, 3))
+    out = {"tau": np.empty(1), "v0": np.empty((n, 3)), "gamma": np.empty(n)}
+    lbp.lbp_adjoint_backward(h, steps, g, None, out)
+    return list(out.values())
+
+
+def free_bytes():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+MB = 1 << 20
+
+
+def test_gradient_memory_is_reused_and_released():
+    """A second gradient takes no more memory and a much smaller one gives the large
+    blocks back; lbp_adjoint_release gives back what is kept, with the recording."""
+    h = handle((64, 64, 64), 6)
+    copy = 64 ** 3 * 60  # bytes of the populations
+    lbp.lbp_step(h, 2)
+    start = free_bytes()
+    gradient(h, 30, 30)
+    one = free_bytes()
+    assert start - one >= 30 * copy  # a checkpoint and 29 states, at least
+    gradient(h, 30, 30)
+    assert free_bytes() == one
+    gradient(h, 4, 4)
+    assert free_bytes() >= one + 20 * copy
+    lbp.lbp_adjoint_release(h)
+    assert free_bytes() >= start - 2 * MB
+    with pytest.raises(lbp.LbpError) as ei:
+        lbp.lbp_adjoint_backward(h, 4, np.ones((4, 6, 3)), None, {"v0": np.empty((6, 3))})
+    assert ei.value.status == lbp.LBP_ESTATE
+    twin = handle((64, 64, 64), 6)  # the same state reached without the gradients in between
+    lbp.lbp_step(twin, 2 + 30 + 30 + 4)
+    assert same(state(h), state(twin))
+    assert same(gradient(h, 8, 3), gradient(twin, 8, 3))
+    lbp.lbp_destroy(h)
+    lbp.lbp_destroy(twin)
+
+
+def test_gradient_memory_does_not_starve_other_handles():
+    """With the device nearly full, a new handle gets the idle block of another's
+    reverse sweep, whose next gradient is the same."""
+    h, twin = handle((128, 128, 128), 4), handle((128, 128, 128), 4)
+    gradient(h, 21, 21)  # keeps about 2.8 GB
+    want = gradient(twin, 21, 21), gradient(twin, 21, 21)
+    lbp.lbp_destroy(twin)
+    torch.cuda.empty_cache()
+    filler = torch.empty(free_bytes() - 1536 * MB, dtype=torch.uint8, device="cuda")
+    assert free_bytes() < 2000 * MB
+    other = lbp.lbp_create(256, 256, 256, 0.8)  # 2 GB
+    lbp.lbp_step(other, 1)
+    lbp.lbp_check(other)
+    lbp.lbp_destroy(other)
+    del filler
+    torch.cuda.empty_cache()
+    assert same(gradient(h, 21, 21), want[1])
+    lbp.lbp_destroy(h)
