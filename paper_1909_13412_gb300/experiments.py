@@ -73,7 +73,6 @@ def pinned_sphere_drag(L, tau, U, R, mode=lbp.LBP_STOKESLET, steps=20000, hold_e
     N = L ** 3
     h = lbp.lbp_create(L, L, L, tau)
     try:
-        lbp.lbp_set_use_graphs(h, False)  # the body force changes every hold_every steps
         u = np.zeros((3, N))
         u[0] = U
         lbp.lbp_set_fluid(h, None, u)
@@ -114,7 +113,6 @@ def kick_and_release(L, tau, M, gamma, R, amplitude, T, t_hold, position=None):
     def run(n_force):
         h = lbp.lbp_create(L, L, L, tau)
         try:
-            lbp.lbp_set_use_graphs(h, False)
             lbp.lbp_particles_add(h, pos, np.zeros((1, 3)), np.array([M]), np.array([gamma]), np.array([R]))
             lbp.lbp_particles_set_params(h, kT=0.0, seed=0)
             V = np.zeros((1, 3))

@@ -41,3 +41,25 @@ def test_chain_is_not_slower_than_plain_launches(precision, shape, n):
     lbp.lbp_set_use_graphs(h, False)
     assert chain <= 1.05 * step_seconds(h)
     lbp.lbp_destroy(h)
+
+
+def test_experiments_run_their_steps_as_a_chain(monkeypatch):
+    """The drag and the kick experiments leave the chain on; their results are those
+    of plain launches, bit for bit."""
+    from paper_1909_13412_gb300 import experiments as ex
+    run = lambda: (ex.pinned_sphere_drag(20, 0.8, 1e-4, 0.4, steps=200), ex.kick_and_release(16, 0.8, 2.0, 0.5, 0.3, 1e-4, 12, 5))
+    switched = []
+    monkeypatch.setattr(ex.lbp, "lbp_set_use_graphs", lambda h, on: switched.append(on))
+    chained = run()
+    assert not any(on is False for on in switched)
+    monkeypatch.undo()
+    create = ex.lbp.lbp_create
+
+    def plain(*args, **kw):
+        h = create(*args, **kw)
+        lbp.lbp_set_use_graphs(h, False)
+        return h
+    monkeypatch.setattr(ex.lbp, "lbp_create", plain)
+    want = run()
+    assert chained[0] == want[0]
+    assert all(np.array_equal(a, b) for a, b in zip(chained[1], want[1]))
