@@ -420,10 +420,11 @@ lbp_status lbp_philox4x64_10(const uint64_t *ctr, const uint64_t *key, uint64_t 
  * samples[t0] * samples[t0 + k], counts[k] = npairs * (T - k) (0 if k >= T),
  * k = 0..max_lag -- the same estimator as lbp_vacf_read.  Products are FP32;
  * the products of one component over one block of at most 64 samples are
- * summed in FP32, every sum above that in FP64.  Scratch is a fixed 4 MiB
- * array inside the library, so ceil(ncomp / 1024) * (max_lag + 1) must not
- * exceed 524288, and ncomp must not exceed 65535 * 1024 (LBP_EINVAL
- * otherwise, with nothing queued).  The first call on a device looks up that
+ * summed in FP32, every sum above that in FP64.  With non-finite samples csum is
+ * non-finite at every lag at which one of them enters a pair, and may be NaN at
+ * others.  Scratch is a fixed 4 MiB array inside the library; the call takes
+ * ceil(ncomp / 1024) * (max_lag + 1) <= 524288 and ncomp <= 65535 * 1024
+ * (LBP_EINVAL otherwise, with nothing queued).  The first call on a device looks up that
  * array's address and keeps it for the life of the process; make it before
  * capturing this routine into a CUDA graph, and do not use this routine on a
  * device after cudaDeviceReset (the kept address would be stale).  All calls

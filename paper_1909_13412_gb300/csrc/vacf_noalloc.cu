@@ -50,7 +50,7 @@ constexpr int NB = 64;       // samples per correlation block
 constexpr int NKT = 128;     // lags per CTA
 constexpr int NLW = 16;      // lags per warp
 constexpr int NJ = 64;       // components per work unit (two per lane)
-constexpr int NJCH = 1024;   // components per scratch row the caller's sizes are checked against
+constexpr int NJCH = 1024;   // components per chunk of the sizes the call takes
 constexpr int NT = 256;      // threads
 constexpr int NWB = 4;       // window blocks in the ring
 constexpr int MAX_RUNS = 512;  // CTAs per lag tile
@@ -224,8 +224,9 @@ extern "C" lbp_status lbp_vacf_correlate_noalloc(const float *samples, int64_t T
     if (!csum || !counts || (T > 0 && !samples))
         return lbp_set_error_for_noalloc(LBP_EINVAL, "lbp_vacf_correlate_noalloc: null pointer");
     const long long nchunks = ((long long)ncomp + NJCH - 1) / NJCH;
-    // both factors are at least 1, so this also bounds max_lag (and with it the
-    // grid sizes below) by the scratch size
+    // the limits of the interface, from a layout with a scratch row per chunk and a
+    // grid row each.  Today's needs max_lag below the scratch size, and with it the
+    // grid sizes below bounded, which follows: both factors are at least 1
     if (nchunks * ((long long)max_lag + 1) > SCRATCH_DOUBLES)
         return lbp_set_error_for_noalloc(
             LBP_EINVAL,

@@ -453,6 +453,8 @@ def lbp_check(h: Handle):
 
 
 def lbp_diagnostics(h: Handle):
+    """fit_per_corner (a name from an earlier layout of the particle kernel): the
+    corners' geometry is prepared before the lattice pass ahead of it ends."""
     out = np.zeros(6, np.int64)
     _call("lbp_diagnostics", h.ptr, C.c_void_p(out.ctypes.data), 6)
     return {"overflow_shares": int(out[0]), "record_slots": int(out[1]), "segments": int(out[2]),
