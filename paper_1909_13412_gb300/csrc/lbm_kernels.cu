@@ -273,7 +273,10 @@ __global__ void __launch_bounds__(BX, R == 2 ? 8 : 1) k_stream_collide_forced(
 // load and store instructions per node and leaves the conversions packed, so
 // the kernel is no longer bound by instruction issue.  Per node the
 // arithmetic is that of collide_st: results equal the one-node kernels'
-// bit for bit.
+// bit for bit.  Its steps are not chained, so its loads could be read-only ones;
+// us per step at 254 x 256 x 256 with 16384 particles, through L2 / read-only: one row
+// BF16 298 / 277, FP16 276 / 278, two rows 264 / 280, 295 / 270 (without particles
+// within 3 % either way): the best of each storage is not slower through L2.
 // ---------------------------------------------------------------------------
 template <typename St>
 __device__ __forceinline__ void unpack2(unsigned v, int a, float &lo, float &hi);
@@ -354,7 +357,7 @@ __global__ void __launch_bounds__(PAIR_BX) k_stream_collide_pair(
         for (int a = 0; a < Q; ++a) {
             const int rb = drow[h] + n.oy[ey(a) + 1] + n.oz[ez(a) + 1];  // source row start
             const unsigned *src = reinterpret_cast<const unsigned *>(pl.s[a] + rb);
-            const unsigned v = __ldcg(src + (x >> 1));  // ahead of the wait: through L2
+            const unsigned v = __ldcg(src + (x >> 1));
             unsigned w = v;
             if (ex(a) > 0) {
                 // pull from x - 1: (x - 1, x) = (hi of left pair, lo of own)
@@ -463,7 +466,7 @@ constexpr int quad_warps(int R) { return R == 1 ? 2 : 4; }
 // With one row the kernel is bound by latency and instruction issue: it is held
 // to 72 registers for 28 warps per SM.  us a step at 256^3 with 16384 particles,
 // BF16 / FP16: 24 warps (80 registers) 206.5 / 222.0, 28 in blocks of four
-// 202.1 / 198.7, in blocks of two 200.9 / 197.6, 30 (64 registers) 213.5 / 211.3.
+// 202.1 / 198.7, in blocks of two 200.9 / 197.6, 32 (64 registers) 213.5 / 211.2.
 // Nothing between the population loads and the record load needs a loaded value
 // (the shuffles of the pull come after), so that the two latencies overlap; a
 // record loaded after the shuffles measured 224.8 / 212.6, and as a read-only load
