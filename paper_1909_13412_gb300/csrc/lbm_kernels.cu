@@ -475,8 +475,14 @@ constexpr int quad_warps(int R) { return R == 1 ? 2 : 4; }
 // cached, unmarked kernel was at 213.0 / 215.3.  More rows keep more loads in
 // flight and need the registers.
 
+// The pass without particles in FP16 is better at 80 registers once the buffers are
+// beyond L2 (BACK: see block_of); us per step, 72 / 80: 7.4 / 8.4 (64^3), 51.5 / 53.2
+// (160^3), 96.3 / 88.6 (200^3), 159.7 / 151.2 (256^3), 354 / 322 (320^3), 699 / 643 (400^3).
+template <typename St, int R, bool FORCED, bool BACK>
+constexpr int QUAD_BLOCKS = R > 1 ? 1 : St::SCALED && !FORCED && !BACK ? 12 : 14;
+
 template <typename St, int R, int MAXR, bool FORCED, bool BACK>
-__global__ void __launch_bounds__(32 * quad_warps(R), R == 1 ? 14 : 1) k_stream_collide_quad(
+__global__ void __launch_bounds__(32 * quad_warps(R), QUAD_BLOCKS<St, R, FORCED, BACK>) k_stream_collide_quad(
     Planes<St> pl, const RepTable<MAXR> rt, const unsigned long long *rec_cur,
     unsigned long long *rec_prev, unsigned long long *fq, long long Ntot, long long *bump, int *err, const Marks mk, bool flip) {
     if (!FORCED && blockIdx.x == 0 && threadIdx.x == 0) *bump += 1;
