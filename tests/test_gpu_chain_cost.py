@@ -55,6 +55,22 @@ def test_two_byte_types_take_the_same_time(edge):
     assert took[1] <= 1.05 * took[0]
 
 
+@pytest.mark.parametrize("edge,n", [(100, 8000), (160, 32768)])
+def test_dense_suspension_in_two_bytes(edge, n):
+    """Half the bytes take no longer than FP32, also where most force records
+    overflow (the four-node kernel took 1.35 times as long here with its
+    accumulators read one by one)."""
+    took = []
+    for precision in (lbp.LBP_F32, lbp.LBP_BF16, lbp.LBP_F16):
+        h = lbp.lbp_create(edge, edge, edge, 0.8, precision=precision)
+        ps = wl.uniform_particles(n, (edge, edge, edge), 10.0, 0.5, 0.26, 1e-4, 5, 6)
+        lbp.lbp_particles_add(h, ps.r, ps.V, ps.M, ps.gamma, ps.R)
+        lbp.lbp_particles_set_params(h, kT=1e-4, seed=3)
+        took.append(step_seconds(h))
+        lbp.lbp_destroy(h)
+    assert max(took[1:]) <= took[0]
+
+
 def test_experiments_run_their_steps_as_a_chain(monkeypatch):
     """The drag and the kick experiments leave the chain on; their results are those
     of plain launches, bit for bit."""

@@ -70,3 +70,16 @@ def test_chained_couplings_on_marked_boxes(boxes, precision, shape, mode, n):
     want = run(*args, [1] * 70, shape=shape, chain=False, mode=mode, lag=20)
     got = run(*args, [70], shape=shape, mode=mode, lag=20)
     assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("boxes", [[(16, 10, 8), (24, 6, 10)], [(24, 3, 5)], [(136, 6, 6)]])
+@pytest.mark.parametrize("precision", [lbp.LBP_BF16, lbp.LBP_F16])
+def test_dense_forces_on_every_shape(boxes, precision):
+    """Several times more force shares than the records hold: every kernel takes its
+    segments' overflow (the two- and four-node ones pairs of it at a time)."""
+    n = 20 * boxes[0][1] * boxes[0][2] // 8
+    want = run(boxes, n, precision, [12], (1, 0), chain=False)
+    shapes = [(2, 0), (1, 1), (2, 1), (4, 1), (1, 2), (1, 3), (2, 3), (4, 3)]
+    for shape in shapes:
+        got = run(boxes, n, precision, [12], shape)
+        assert all(np.array_equal(a, b) for a, b in zip(got, want)), shape

@@ -103,8 +103,11 @@ def test_force_overflow_is_read_through_l2(name, file):
     body = kernel(name, file)
     reads = re.findall(r"[^\n;]*\bfqd?\s*(?:\[|\+)[^;]*;", body)
     reads = [r for r in reads if not re.search(r"\bfqd?\s*\[[^=]*\]\s*=[^=]", r)]
-    assert reads or "__ldcg(fq" in body
-    assert all("__ldcg(fq" in r for r in reads), reads
+    through_l2 = ("__ldcg(fq", "take_shares(fq")  # a volatile asm, and one on a pair of them
+    assert reads and all(any(f in r for f in through_l2) for r in reads), reads
+    helper = source("lbm_kernels.cu")
+    helper = block(helper, helper.index("take_shares("))
+    assert "__ldcg(at)" in helper and volatile_ldcg(cuda_headers(), "ulonglong2")
 
 
 def test_exchange_asks_for_a_buffers_attributes_once():
