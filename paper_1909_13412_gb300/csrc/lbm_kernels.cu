@@ -304,18 +304,6 @@ __device__ __forceinline__ unsigned pack2<StoreF16>(float lo, float hi, int) {
     return *reinterpret_cast<const unsigned *>(&p);
 }
 
-// Read and clear the overflow accumulators of a node pair (through L2: the particle
-// kernels' atomics add to them).  16-byte aligned: these kernels need even rows in
-// every box, so planes and rows start at even nodes.  One by one, a four-node lane made
-// twelve 8-byte loads and stores: us per step with 8 particles per 1000 nodes, BF16,
-// 100^3 72 -> 38, 160^3 390 -> 224, 256^3 1128 -> 726.
-__device__ __forceinline__ ulonglong2 take_shares(unsigned long long *fq) {
-    ulonglong2 *at = reinterpret_cast<ulonglong2 *>(fq);
-    const ulonglong2 v = __ldcg(at);
-    *at = make_ulonglong2(0ull, 0ull);
-    return v;
-}
-
 constexpr int PAIR_BX = SEG / 2;  // threads per block of the paired kernel
 
 // True if either 2-byte value of a packed pair is a NaN or an infinity (its
@@ -409,9 +397,10 @@ __global__ void __launch_bounds__(PAIR_BX) k_stream_collide_pair(
                     const int d = drow[h] + x;
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        const ulonglong2 v = take_shares(fq + k * Ntot + d);
-                        s0[k] += (long long)v.x;
-                        s1[k] += (long long)v.y;
+                        s0[k] += (long long)__ldcg(fq + k * Ntot + d);
+                        s1[k] += (long long)__ldcg(fq + k * Ntot + d + 1);
+                        fq[k * Ntot + d] = 0ull;
+                        fq[k * Ntot + d + 1] = 0ull;
                     }
                 }
                 const float inv = 1.3877787807814457e-17f;  // 2^-56
@@ -432,6 +421,19 @@ __global__ void __launch_bounds__(PAIR_BX) k_stream_collide_pair(
                 reinterpret_cast<unsigned *>(pl.d[a] + drow[h])[x >> 1] = pack2<St>(o0[a], o1[a], a);
         }
     }
+}
+
+// Read and clear the overflow accumulators of a node pair (through L2: the particle
+// kernels' atomics add to them).  16-byte aligned: the four-node kernel needs rows of
+// a multiple of four in every box, so planes, rows and pairs start at even nodes.  One
+// by one, a lane made twelve 8-byte loads and stores: us per step with 8 particles per
+// 1000 nodes, BF16, 100^3 72 -> 38, 160^3 390 -> 224, 256^3 1128 -> 726.  (In the two-node
+// kernel pairs cost registers: 254 x 256 x 256, BF16, two rows 265 -> 281; not used there.)
+__device__ __forceinline__ ulonglong2 take_shares(unsigned long long *fq) {
+    ulonglong2 *at = reinterpret_cast<ulonglong2 *>(fq);
+    const ulonglong2 v = __ldcg(at);
+    *at = make_ulonglong2(0ull, 0ull);
+    return v;
 }
 
 // Sum, exactly, the record entries whose x is one of x .. x + 3 (one pass
